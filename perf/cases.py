@@ -261,6 +261,29 @@ def run(s):
     return out
 
 
+# ------------------------------------------------------------------------------------ in 64 bits --
+def exact(case, seed):
+    """H and diag((H + damp I)^-1) in 64 bits.  Codes, grids and losses have no entry: a weight within fp32 rounding of a
+    midpoint goes either way and takes the rest of its row along, so what they are off by is luck and not precision (the
+    tolerance below bounds it); an activation-ordered layer has its dinv in an order that rounding of H decides."""
+    kind, c, n = case["kind"], case.get("c", 0), case.get("n", 0)
+    if kind in ("stack", "record") or c > 16384 or case.get("act_order"):
+        return None
+    dtype = torch.float32 if case.get("dtype") == "fp32" else torch.bfloat16
+    X = _inputs(c, n, seed, 0, dtype, "low_rank" if kind == "calib" else case["inputs"], token_major=kind == "calib")
+    H = torch.zeros((c, c), device="cuda", dtype=torch.float64)
+    for j in range(0, n, 16384):
+        x = X[j:j + 16384].t().double() if kind == "calib" else X[:, j:j + 16384].double()
+        H.addmm_(x, x.t(), alpha=2.0)
+    if kind == "calib":
+        return H
+    H.diagonal().add_(0.01 * H.diagonal().mean())
+    R_inv = torch.linalg.solve_triangular(torch.linalg.cholesky(H), torch.eye(c, device="cuda", dtype=torch.float64), upper=False)
+    out = dict(codes=None, loss=None, dinv=R_inv.square_().sum(dim=0))
+    out.update(dict(grid=None) if case["grid"] == "nonuniform" else dict(scale=None, zero=None))
+    return out
+
+
 # ------------------------------------------------------------------------------- floors, limits --
 def _layer_work(r, c, n, elem, K, exact=False):
     """X and W read, codes and tables written; X X^T by symmetry, the factor of the inverse, the column loop's updates."""
