@@ -67,6 +67,35 @@ def test_record_affine_bit_exact(lq, h, r, c, bits, group):
     assert np.array_equal(f64(back), O.unpack_layer(want))
 
 
+@pytest.mark.parametrize("grid,bits,c,group", [("nonuniform", 2, 8, 0), ("nonuniform", 3, 1032, 0), ("nonuniform", 4, 1024, 0),
+                                               ("nonuniform", 3, 32, 0), ("affine", 3, 40, 8), ("affine", 2, 2080, 16),
+                                               ("affine", 4, 36, 12)])
+@pytest.mark.parametrize("dtype,pad,shift", [(torch.bfloat16, 0, 0), (torch.float32, 8, 0), (torch.bfloat16, 8, 0), (torch.float32, 0, 1),
+                                             (torch.bfloat16, 3, 0)])
+def test_record_unpacks_at_unit_edges(lq, h, grid, bits, c, group, dtype, pad, shift):
+    """Widths at the edges of a unit (8, 32 codes) and of a warp's 1024 weights, strided and misaligned output rows: the
+    wide kernels and the general ones give the same values, and what lies between the output rows stays untouched."""
+    r = 11
+    g = torch.Generator().manual_seed(c + bits)
+    codes = torch.randint(0, 256, (r, c), generator=g, dtype=torch.uint8)         # bits above the b-bit code are cut off
+    cfg = lq.Config.make(grid=grid, bits=bits, group=group, T=45, t=9)
+    kw = {}
+    if grid == "affine":
+        kw = dict(scale=torch.rand(r, c // group, generator=g) * 0.01 + 1e-4,
+                  zero=torch.randint(-4, 1 << bits, (r, c // group), generator=g, dtype=torch.int32))
+    else:
+        kw = dict(grid=torch.sort(torch.randn(r, 1 << bits, generator=g) * 0.03, dim=1).values)
+    rec = lq.lq_pack_layer(h, cfg, codes.cuda(), **{k: v.cuda() for k, v in kw.items()})
+    want = O.pack_layer(codes.numpy() & ((1 << bits) - 1), bits, **{k: v.numpy() for k, v in kw.items()}, **(dict(group=group) if group else {}))
+    assert np.array_equal(rec.cpu().numpy(), want)
+    buf = torch.full((r * (c + pad) + shift,), 7.0, dtype=dtype, device="cuda")
+    out = buf[shift:].view(r, c + pad)[:, :c]
+    lq.lq_unpack_layer(h, cfg, rec, r, c, out)
+    lq.lq_sync_status(h)
+    assert torch.equal(out.cpu(), torch.from_numpy(O.unpack_layer(want)).to(torch.float32).to(dtype))
+    assert bool((buf[shift:].view(r, c + pad)[:, c:] == 7.0).all()) and bool((buf[:shift] == 7.0).all())
+
+
 def test_record_zero_point_out_of_range_is_reported(lq, h):
     codes = torch.zeros(2, 64, dtype=torch.uint8, device="cuda")
     scale = torch.ones(2, 1, device="cuda")
