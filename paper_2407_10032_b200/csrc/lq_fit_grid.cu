@@ -902,19 +902,75 @@ affine_search_warp_kernel(const T* __restrict__ W, int64_t ldw, int group, int n
 // constant u the ratio lo / S grows by (K - 1) / (T - u) per step of t_min, so Z = -rint(lo / S)
 // keeps one integer value over a run of about (T - u) / (K - 1) consecutive candidates: at the
 // paper's T = 2048 the (t + 1)^2 = 168100 candidates of the 4-bit search give only ~2400
-// different grids.  This kernel scores each class (u, Z) once, in fp32, and evaluates in fp64,
+// different grids.  This kernel scores classes (u, Z) in fp32 and evaluates in fp64,
 // with the arithmetic of Eq. 7, only the first member (in t_min-major order) of every class whose
 // score lies within 0.1 % of the best; the arg-min is the lexicographic minimum of (fp64 loss,
-// candidate index) over those.  The members of a class have fp64 losses that differ by rounding
+// candidate index) over those.
+//
+// Most classes need no score.  With the weights as a vector in the norm sqrt(sum_j s_j x_j^2), f(S, Z) = sqrt(loss) is the
+// distance of the weights from the grid, and moving the grid moves f by no more than the norm of the points' shifts: if
+// m'_j = (index - Z) of the point nearest w_j on the grid (S', Z), then dist_j(S') = |w_j - m'_j S'| >= |w_j - m'_j S| -
+// |m'_j| |S' - S| >= dist_j(S) - |m'_j| |S' - S|, hence f(S', Z) >= f(S, Z) - |S' - S| B with B = sqrt(sum_j s_j m'_j^2).
+// Where Z lies in [0, K - 1] the clamp moves an index towards zero, so |m'_j| <= |w_j| / S' + 1/2, and in any case
+// |m'_j| <= max(|Z|, |K - 1 - Z|): B follows from three sums over the group.  So the lines of constant u are taken in blocks
+// of AC_BLOCK, one line of a block (its anchor) is scored for every Z that occurs in the block, and a class of another line
+// is scored only if the bound from its anchor does not put it above the bar (aff_bar32 of the best valid anchor, which
+// is no lower than the final one; the fp32 errors of the scores are taken off as in aff_bar32).  At T = 2048 about 300 of
+// 2400 classes are scored at 4 bits (blocks of 8 lines: 380, of 32: more survive), and the classes that are left out could
+// not have been listed for fp64: the result is the same.  4096 x 4096 in groups of 128, 4 bits: 15.7 -> 5.8 ms; what is
+// left is instruction issue (66 % of the slots): scores, the set-up of 819 lines and ~10 classes in fp64.  The members of a class have fp64 losses that differ by rounding
 // noise only, so this is the all-candidate search up to which member of the winning class is
 // named (same Z, S equal to ~1e-16).
 // One CTA per group.  Requires (K - 1) / (T - 2t) < 1/2: then every integer between the Z of the
 // two ends of a line is taken by some candidate on it.
 constexpr int AC_MAX_U = 2048;           // lines of constant u: 2t + 1 of them
 constexpr int AC_MAX_THREADS = 512;
+constexpr int AC_BLOCK = 16;
+constexpr long long AC_MIN_WORK = 65536;         // classes x weights of a group from which on classes are left out
+constexpr int AC_MAX_BLOCKS = AC_MAX_U / AC_BLOCK + 1;
+
+// Loss of Eq. 7 of one candidate over a group, by a warp (lane l takes weights l, l + 32, ... in that order).  rint(w / S)
+// comes from the reciprocal: w / S rounded and w (1 / S) differ by less than 2^-51 |w / S|, so further than 1e-12 of that from
+// a tie both round to the same integer; only a lane that holds a weight nearer to a tie (or an infinity or NaN) divides.  Four
+// weights at a time keep four loads and four chains of fp64 operations in flight: one at a time, a long group is bound by
+// their latency (14336 weights per row, 2 bits, T = 2048: 25 ms per 64 rows).
+template <typename WAt>
+__device__ __forceinline__ double aff_loss64(WAt w_at, const double* __restrict__ sp, int group, double S, double Z, double Km1, int lane) {
+    const double rS = 1.0 / S;
+    double loss = 0.0;
+    for (int j0 = lane; j0 < group; j0 += 128) {
+        double w[4], s[4], q[4];
+        bool near_tie = false;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool in = j0 + 32 * e < group;
+            w[e] = in ? static_cast<double>(w_at(j0 + 32 * e)) : 0.0;
+            s[e] = in ? LQ_AT(sp + j0 + 32 * e) : 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double t = w[e] * rS;
+            q[e] = rint(t);
+            near_tie |= !(fabs(t - q[e]) < 0.5 - 1e-12 * (1.0 + fabs(t)));
+        }
+        if (near_tie) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) q[e] = rint(w[e] / S);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double k = fmin(fmax(q[e] + Z, 0.0), Km1);
+            const double d = (k - Z) * S - w[e];
+            if (j0 + 32 * e < group) loss += s[e] * (d * d);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    return loss;
+}
 
 template <typename T>
-__global__ void __launch_bounds__(AC_MAX_THREADS)
+__global__ void __launch_bounds__(AC_MAX_THREADS, 2)
 affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_groups, const double* __restrict__ s64, int K,
                     int Tparts, int t_count, int p_max, float* __restrict__ scale, int32_t* __restrict__ zero, int64_t out_ld,
                     lq_dev_status* __restrict__ dstatus) {
@@ -923,12 +979,14 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
     float2* ws = reinterpret_cast<float2*>(ac_smem);                          // (w - min, s / max s) of the group
     int* off = reinterpret_cast<int*>(ws + group);                             // nu + 1: first class of each line
     int* za = off + nu + 1;                                                    // nu: Z at the first candidate of the line
-    float* score = reinterpret_cast<float*>(za + nu);                          // p_max
-    int* list = reinterpret_cast<int*>(score + p_max);                         // p_max: classes to evaluate in fp64
-    __shared__ double red_d[AC_MAX_THREADS / 32], red_s[AC_MAX_THREADS / 32];
+    float* score = reinterpret_cast<float*>(za + nu);                          // p_max: of the anchors, then of the listed classes
+    uint16_t* list = reinterpret_cast<uint16_t*>(score + p_max);               // p_max: classes to score
+    uint16_t* list64 = list + p_max;                                           // p_max: entries of `list` to evaluate in fp64
+    __shared__ int ab_off[AC_MAX_BLOCKS + 1], ab_z0[AC_MAX_BLOCKS];            // first anchor and highest Z of each block of lines
+    __shared__ double red_d[AC_MAX_THREADS / 32], red_s[AC_MAX_THREADS / 32], red_1[AC_MAX_THREADS / 32], red_2[AC_MAX_THREADS / 32];
     __shared__ float red_f[2][AC_MAX_THREADS / 32];
     __shared__ int red_i[AC_MAX_THREADS / 32];
-    __shared__ int n_list;
+    __shared__ int n_list, n_list64;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarp = nthr >> 5;
     const int64_t gid = blockIdx.x;
@@ -939,13 +997,16 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
     const double* sp = s64 + static_cast<int64_t>(gi) * group;
 
     float mn = INFINITY, mx = -INFINITY;
-    double smax = 0.0, ssum = 0.0;
+    double smax = 0.0, ssum = 0.0, s1 = 0.0, s2 = 0.0;           // s1, s2: sum s |w|, sum s w^2
     for (int j = tid; j < group; j += nthr) {
         const float w = load_w(wp + j);
+        const double sj = LQ_AT(sp + j), sw = sj * fabs(static_cast<double>(w));
         mn = fminf(mn, w);
         mx = fmaxf(mx, w);
-        smax = fmax(smax, LQ_AT(sp + j));
-        ssum += LQ_AT(sp + j);
+        smax = fmax(smax, sj);
+        ssum += sj;
+        s1 += sw;
+        s2 += sw * fabs(static_cast<double>(w));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -953,13 +1014,16 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
         ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
-    if (lane == 0) { red_f[0][warp] = mn; red_f[1][warp] = mx; red_d[warp] = smax; red_s[warp] = ssum; }
-    if (tid == 0) n_list = 0;
+    if (lane == 0) { red_f[0][warp] = mn; red_f[1][warp] = mx; red_d[warp] = smax; red_s[warp] = ssum; red_1[warp] = s1; red_2[warp] = s2; }
+    if (tid == 0) n_list = n_list64 = 0;
     __syncthreads();
-    ssum = 0.0;
+    ssum = s1 = s2 = 0.0;
     for (int w = 0; w < nwarp; ++w) {
         mn = fminf(mn, red_f[0][w]); mx = fmaxf(mx, red_f[1][w]); smax = fmax(smax, red_d[w]); ssum += red_s[w];
+        s1 += red_1[w]; s2 += red_2[w];
     }
     __syncthreads();                                  // the scratch is reused below
     const double sinv = smax > 0.0 ? 1.0 / smax : 1.0;
@@ -991,11 +1055,20 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
     };
 
     // classes per line of constant u, then their exclusive prefix sum
+    const double step = R / dT;
     for (int u = tid; u < nu; u += nthr) {
         const int a = max(0, u - t_count), b = min(t_count, u);
         double Sa, Za, Sb, Zb;
         int cnt = 0, z0 = 0;
-        if (params(a, u - a, Sa, Za) && params(b, u - b, Sb, Zb) && fabs(Za) < 1e9 && fabs(Zb) < 1e9) {
+        // Z of the two end candidates with one division instead of six.  With X = (|min| + R) / S the quotients here and in
+        // Eq. 7's expressions are off by a few 2^-53 X, plus 2^-53 X |min| / (R (1 - u / T)) through the cancellation in
+        // Eq. 7's S: below 1e-9 X (1 + 1e-6 X), and an estimate further than that from a tie rounds as they do
+        const double rS = Km1 / (step * static_cast<double>(Tparts - u));
+        const double qa = fma(static_cast<double>(a), step, dmn) * rS, qb = fma(static_cast<double>(b), step, dmn) * rS;
+        Za = -rint(qa); Zb = -rint(qb);
+        const double X = 1.0 + (fabs(dmn) + R) * rS, tie = 0.5 - 1e-9 * X * (1.0 + 1e-6 * X);
+        const bool sure = fabs(qa + Za) < tie && fabs(qb + Zb) < tie;          // false for NaN and infinities too
+        if ((sure || (params(a, u - a, Sa, Za) && params(b, u - b, Sb, Zb))) && fabs(Za) < 1e9 && fabs(Zb) < 1e9) {
             z0 = static_cast<int>(Za);
             cnt = max(z0 - static_cast<int>(Zb), 0) + 1;
         }
@@ -1040,34 +1113,123 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
     const double c_s = R / (dT * Km1);               // S of line u = c_s (T - u)
     const float Km1f = static_cast<float>(K - 1);
 
-    // fp32 score of every class
+    const float Rf = static_cast<float>(R);
+
+    // Where scoring everything is little work (short groups, few classes) it is faster than two rounds of scores with
+    // barriers between them: the line is between 256 groups of 32 at T = 1000 (P g = 38 000: 0.30 against 0.36 ms) and of 64
+    // at T = 2048 (150 000: 0.35 against 0.25 ms).
+    const int n_blk = (nu + AC_BLOCK - 1) / AC_BLOCK;
+    int n_anchor = 0;
+    bool prune = static_cast<long long>(P) * group >= AC_MIN_WORK;
+    if (prune) {
+        // highest Z and number of anchors of each block of lines, then the exclusive prefix sum
+        for (int i = tid; i < n_blk; i += nthr) {
+            int zh = -0x7fffffff, zl = 0x7fffffff;
+            for (int u = AC_BLOCK * i; u < min(AC_BLOCK * (i + 1), nu); ++u) {
+                const int cnt = LQ_AT(off + u + 1) - LQ_AT(off + u);
+                if (cnt > 0) { zh = max(zh, LQ_AT(za + u)); zl = min(zl, LQ_AT(za + u) - cnt + 1); }
+            }
+            ab_z0[i] = zh;
+            ab_off[i] = zh >= zl ? min(zh - zl + 1, p_max + 1) : 0;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int base = 0;
+            for (int i0 = 0; i0 < n_blk; i0 += 32) {
+                const int v = i0 + lane < n_blk ? ab_off[i0 + lane] : 0;
+                int incl = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                __syncwarp();
+                if (i0 + lane < n_blk) ab_off[i0 + lane] = base + incl - v;
+                base += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) ab_off[n_blk] = base;
+        }
+        __syncthreads();
+        n_anchor = ab_off[n_blk];
+        // a group far from zero (|Z| in the hundreds, drifting along u) may have more anchors than there is room for, or as
+        // many as classes: then every class is scored
+        prune = n_anchor <= p_max && 2 * n_anchor <= P;
+    }
+    if (prune) {
+        float best_a = INFINITY;
+        for (int q = tid; q < n_anchor; q += nthr) {
+            int lo_b = 0, hi_b = n_blk - 1;
+            while (lo_b < hi_b) {                    // the last block whose first anchor is <= q
+                const int mid = (lo_b + hi_b + 1) >> 1;
+                if (ab_off[mid] <= q) lo_b = mid; else hi_b = mid - 1;
+            }
+            const int u = min(AC_BLOCK * lo_b + AC_BLOCK / 2, nu - 1), Zi = ab_z0[lo_b] - (q - ab_off[lo_b]);
+            const AffScore as = aff_score_setup(c_s * static_cast<double>(Tparts - u), static_cast<double>(Zi), dmn, Km1);
+            const float sc = aff_score32(ws, group, as, Km1f);
+            LQ_AT(score + q) = sc;
+            const int k = LQ_AT(za + u) - Zi;
+            if (k >= 0 && k < LQ_AT(off + u + 1) - LQ_AT(off + u)) best_a = fminf(best_a, sc);       // the anchor is a class itself
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best_a = fminf(best_a, __shfl_xor_sync(0xffffffffu, best_a, o));
+        if (lane == 0) red_f[0][warp] = best_a;
+        __syncthreads();
+        for (int w = 0; w < nwarp; ++w) best_a = fminf(best_a, red_f[0][w]);
+        // f of an anchor less what its fp32 score and that of the class compared with the bar may be off by: delta
+        // sqrt(sum_s) each, 0.1 % of the loss each (see aff_bar32), and room for the roundings of this bound itself
+        const float slack = 3.0f * 2.2e-7f * Rf * sqrtf(sum_s);
+        const float root_bar = sqrtf(aff_bar32(best_a, Rf, sum_s)) * 1.002f;
+        const float f1 = static_cast<float>(s1 * sinv), f2 = static_cast<float>(s2 * sinv), root_s = sqrtf(sum_s);
+        for (int u = tid; u < nu; u += nthr) {
+            const int p0 = LQ_AT(off + u), cnt = LQ_AT(off + u + 1) - p0, z0 = LQ_AT(za + u);
+            const int blk = u / AC_BLOCK, ua = min(AC_BLOCK * blk + AC_BLOCK / 2, nu - 1);
+            const float S = static_cast<float>(c_s * static_cast<double>(Tparts - u));
+            const float dS = static_cast<float>(c_s) * fabsf(static_cast<float>(u - ua)) * 1.001f;
+            const float rS = 1.0f / S;
+            const float shift = dS * sqrtf(fmaf(fmaf(f2, rS, f1), rS, 0.25f * sum_s));
+            for (int k = 0; k < cnt && p0 + k < P; ++k) {
+                const int Zi = z0 - k;
+                float sh = dS * root_s * static_cast<float>(max(abs(Zi), abs(K - 1 - Zi)));
+                if (Zi >= 0 && Zi <= K - 1) sh = fminf(sh, shift);
+                const float low = sqrtf(LQ_AT(score + ab_off[blk] + (ab_z0[blk] - Zi))) * 0.998f - slack - sh;
+                if (!(low > root_bar)) LQ_AT(list + atomicAdd(&n_list, 1)) = static_cast<uint16_t>(p0 + k);       // NaN: scored
+            }
+        }
+    } else {
+        for (int p = tid; p < P; p += nthr) LQ_AT(list + p) = static_cast<uint16_t>(p);
+        if (tid == 0) n_list = P;
+    }
+    __syncthreads();
+    const int n_score = n_list;
+
+    // fp32 score of every listed class
     float best32 = INFINITY;
-    for (int p = tid; p < P; p += nthr) {
+    for (int i = tid; i < n_score; i += nthr) {
         int u, Zi;
-        class_of(p, u, Zi);
+        class_of(LQ_AT(list + i), u, Zi);
         const AffScore as = aff_score_setup(c_s * static_cast<double>(Tparts - u), static_cast<double>(Zi), dmn, Km1);
         float sc = aff_score32(ws, group, as, Km1f);
         if (sc != sc) sc = -INFINITY;                // a NaN score is always re-examined in fp64
-        LQ_AT(score + p) = sc;
+        LQ_AT(score + i) = sc;
         best32 = fminf(best32, sc == -INFINITY ? INFINITY : sc);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best32 = fminf(best32, __shfl_xor_sync(0xffffffffu, best32, o));
-    if (lane == 0) red_f[0][warp] = best32;
+    if (lane == 0) red_f[1][warp] = best32;
     __syncthreads();
-    for (int w = 0; w < nwarp; ++w) best32 = fminf(best32, red_f[0][w]);
-    const float bar32 = aff_bar32(best32, static_cast<float>(R), sum_s);
-    for (int p = tid; p < P; p += nthr)
-        if (LQ_AT(score + p) <= bar32) LQ_AT(list + atomicAdd(&n_list, 1)) = p;
+    for (int w = 0; w < nwarp; ++w) best32 = fminf(best32, red_f[1][w]);
+    const float bar32 = aff_bar32(best32, Rf, sum_s);
+    for (int i = tid; i < n_score; i += nthr)
+        if (LQ_AT(score + i) <= bar32) LQ_AT(list64 + atomicAdd(&n_list64, 1)) = LQ_AT(list + i);
     __syncthreads();
-    const int n_eval = n_list;
+    const int n_eval = n_list64;
 
     // fp64 loss of the first member of each listed class, one class per warp at a time
     double my_loss = INFINITY;
     int my_idx = 0x7fffffff;
     for (int i = warp; i < n_eval; i += nwarp) {
         int u, Zi;
-        class_of(LQ_AT(list + i), u, Zi);
+        class_of(LQ_AT(list64 + i), u, Zi);
         const int a = max(0, u - t_count), b = min(t_count, u);
         const double Zd = static_cast<double>(Zi);
         // first t_min on the line with rint(lo / S) >= -Z, i.e. with Z(t_min) <= Z: estimate, then settle exactly
@@ -1082,16 +1244,7 @@ affine_class_kernel(const T* __restrict__ W, int64_t ldw, int group, int n_group
             if (params(tm, u - tm, S, Z) && Z > Zd) ++tm; else break;
         }
         if (!params(tm, u - tm, S, Z) || Z != Zd) continue;       // no candidate of the line has this Z
-        double loss = 0.0;
-        for (int j = lane; j < group; j += 32) {
-            const double w = static_cast<double>(load_w(wp + j));
-            double q = rint(w / S) + Z;
-            q = fmin(fmax(q, 0.0), Km1);
-            const double d = (q - Z) * S - w;
-            loss += LQ_AT(sp + j) * (d * d);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        const double loss = aff_loss64([&](int j) { return load_w(wp + j); }, sp, group, S, Z, Km1, lane);
         const int idx = tm * side + (u - tm);
         if (loss < my_loss || (loss == my_loss && idx < my_idx)) { my_loss = loss; my_idx = idx; }
     }
@@ -1123,7 +1276,7 @@ bool affine_class_plan(int K, int Tparts, int t_count, int64_t g, int* p_max, si
     }
     const size_t bytes = static_cast<size_t>(g) * sizeof(float2) + static_cast<size_t>(2 * nu + 1) * sizeof(int) +
                          static_cast<size_t>(total) * (sizeof(float) + sizeof(int));
-    if (bytes > 200 * 1024) return false;
+    if (bytes > 200 * 1024 || total > 65535) return false;       // the lists hold 16-bit class numbers
     *p_max = static_cast<int>(total);
     *smem = bytes;
     return true;
@@ -1180,7 +1333,9 @@ int lq_affine_search(lq_handle* h, cudaStream_t st, const void* W, int32_t w_dty
             LQ_CUDA_TRY(cudaFuncSetAttribute(affine_class_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
         }
         const unsigned nb = static_cast<unsigned>(r * n_groups);
-        const int threads = g > 8192 ? 512 : 256;
+        // ~200 anchors and ~100 survivors per group; 128 threads gain 5 % at 4 bits and lose 50 % at 2 and 3 bits, where the
+        // longer lists leave fewer CTAs per SM; long groups have hundreds of classes to evaluate in fp64 and want the warps
+        const int threads = g > 8192 ? AC_MAX_THREADS : 256;
         if (w_dtype == LQ_F32)
             affine_class_kernel<float><<<nb, threads, smem_c, st>>>(static_cast<const float*>(W), ldw, (int)g, n_groups, s64, K, T,
                                                                    t_count, p_max, scale, zero, out_ld, h->dstatus);

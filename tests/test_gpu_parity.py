@@ -410,6 +410,23 @@ def test_stage3_affine_fine_partition(lq, h, r, c, bits, group, T, t, recipe):
     assert frac >= 0.98
 
 
+@pytest.mark.parametrize("offset,group,T,t", [(0.1, 128, 1024, 250), (-40.0, 256, 1024, 250), (0.0, 64, 2048, 409), (0.0, 1026, 512, 100)])
+def test_stage3_affine_classes_left_out(lq, h, offset, group, T, t):
+    """Groups that hold no zero (Z outside the grid, drifting along the lines of constant t_min + t_max), far-off groups
+    (more anchors than classes: nothing is left out) and group lengths off the vector widths."""
+    g = torch.Generator().manual_seed(group + T)
+    W = torch.randn(2, group, generator=g) * 0.02 + offset
+    dinv32 = torch.exp(torch.randn(group, generator=g))
+    So, Zo = O.fit_grid_affine(f64(W), f64(dinv32), 4, 4.0, group, T, t)
+    cfg = lq.Config.make(grid="affine", bits=4, p=4.0, group=group, T=T, t=t)
+    scale = torch.empty(2, 1, device="cuda")
+    zero = torch.empty(2, 1, dtype=torch.int32, device="cuda")
+    ws = ws_for(lq, lq.lq_fit_grid_workspace(cfg, 2, group))
+    lq.lq_fit_grid(h, cfg, W.cuda(), dinv32.cuda(), ws, scale=scale, zero=zero)
+    lq.lq_sync_status(h)
+    assert _check_affine_picks(f64(W), f64(dinv32), 4, group, T, t, f64(scale), zero.cpu().numpy(), So, Zo) >= 0.98
+
+
 def test_stage3_affine_constant_group(lq, h):
     W = torch.full((2, 128), 0.25)
     W[1] = 0.0
