@@ -2,12 +2,25 @@
 // full downdate of its own copy of the inverse Hessian (Eq. 3 for the weights, Eq. 9 for the inverse).
 //
 // One CTA per row, fp64 throughout (the decisions -- which weight next, which grid point -- must be
-// those of a float64 evaluation).  The row's c x c inverse lives in global memory; the O(c^2)
-// downdate of Eq. 9 is not applied after every step but every `nb` steps: the columns v_m taken out
-// by the steps of the current batch stay in shared memory, the column that a step needs is
+// those of a float64 evaluation).  The O(c^2) downdate of Eq. 9 is not applied after every step but every
+// `nb` steps: the columns v_m taken out by the steps of the current batch stay in shared memory, the column
+// that a step needs is
 //     Hinv_now[:, i] = Hinv_batch_start[:, i] - sum_m v_m (v_m[i] / pivot_m),
 // and a batch ends with one rank-nb update of the matrix, which cuts its memory traffic by nb.
 // The diagonal, which the greedy choice reads at every step, is kept up to date separately.
+//
+// The rows' matrices do not fit the L2 (296 CTAs x 4.7 MB at c = 768), so their traffic is what bounds the kernel, and the
+// layout is made for it.  The weights still to do are kept compact: a batch's update reads the upper triangle of the n
+// weights that the batch started with and writes the one of the n - nb that are left, packed, into the other half of
+// the row's slot (two packed triangles of c - 1 and fewer fill no more than c x c).  The shared memory for the batch's columns holds
+// more of them as n falls: nb grows.  Together n^2 / 2 entries per batch instead of n c / 2 at a fixed nb: c^3 / 7 bytes
+// per row and weight where the loop over all columns moved 2 c^3 / 7.  The first batch reads U^T U itself, which all rows share.
+// The update itself runs on the FP64 MMA (a column of the batch is a step of K): an eighth of the instructions of the same
+// multiply-adds, which were six tenths of the kernel's issue slots.  A step needs one barrier, and what it can do before its
+// column has arrived it does: the pivot is the maintained diagonal, the batch's downdates are summed on their own.
+// 768 x 768, 4 bits: 37.2 -> 19.8 ms (compaction 27.4, MMA and the shorter step 21.7, asking for strips ahead 20.5, bisection and
+// one quantisation per offer 19.8); 23 GB of DRAM traffic per 296 rows where it was 50.  What is left is the latency of a
+// step's column and three rounds of 296 rows for 768.
 #include <cstdint>
 
 #include "lq_common.cuh"
@@ -55,12 +68,15 @@ struct ExactArgs {
     double* loss_rows;            // r
     lq_dev_status* dstatus;
     size_t slot_stride;           // doubles between two copies
-    int64_t r; int c; int K; int nb;
+    int64_t r; int c; int K;
+    int vcap;                     // doubles of shared memory for the columns of a batch
 };
 
-// Nearest grid point by the midpoint rule (the number of midpoints strictly below w), or quant_aff.
+// Nearest grid point by the midpoint rule (the number of midpoints strictly below w: found by bisection where they ascend,
+// as fitted grids do), or quant_aff.
 template <bool AFFINE>
-__device__ __forceinline__ void ex_quant(double w, const double* __restrict__ gpts, int K, double S, double Z, int& code, double& q) {
+__device__ __forceinline__ void ex_quant(double w, const double* __restrict__ gpts, const double* __restrict__ mids, bool ascending, int K,
+                                         double S, double Z, int& code, double& q) {
     if (AFFINE) {
         double t = rint(w / S) + Z;
         t = fmin(fmax(t, 0.0), static_cast<double>(K - 1));
@@ -68,156 +84,212 @@ __device__ __forceinline__ void ex_quant(double w, const double* __restrict__ gp
         q = (t - Z) * S;
     } else {
         int a = 0;
-        for (int k = 0; k + 1 < K; ++k) a += (w > 0.5 * (gpts[k] + gpts[k + 1])) ? 1 : 0;
+        if (ascending) {
+            for (int h = K >> 1; h > 0; h >>= 1) a += (w > mids[a + h - 1]) ? h : 0;
+        } else {
+            for (int k = 0; k + 1 < K; ++k) a += (w > mids[k]) ? 1 : 0;
+        }
         code = a;
         q = gpts[a];
     }
 }
 
-constexpr int EX_PER = 32;      // weights per thread at most (c <= EX_THREADS * EX_PER)
+constexpr int EX_MAX_PER = 32;      // weights per thread at most
+constexpr int EX_MAX_C = 7465;      // widest row: its values, diagonals and one column of a batch fill the shared memory
+constexpr int EX_DONE = 0x8000;     // flag beside the name of a weight
+static_assert(EX_MAX_C <= EX_THREADS * EX_MAX_PER && EX_MAX_C < EX_DONE, "positions");
 
-template <typename T, bool AFFINE>
+// Distance of the batch's columns: 2 modulo 4, so that the 4 x 8 operand tiles of the MMA meet 32 different banks.
+__host__ __device__ __forceinline__ int ex_pitch(int n) { return ((n + 1) & ~3) + 2; }
+// Entries of the space that the list of old positions shares with the warps' coefficients.
+__host__ __device__ __forceinline__ int ex_names(int c) {
+    constexpr int least = EX_WARPS * EX_MAX_NB * 4;
+    return c > least ? (c + 3) & ~3 : least;
+}
+__device__ __forceinline__ void ex_dmma(double& c0, double& c1, double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                 : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
+}
+
+// Start of row p of the packed upper triangle of an n x n matrix, less p: entry (p, q) is at ex_row(p, n) + q.
+__device__ __forceinline__ uint32_t ex_row(int p, int n) {
+    return static_cast<uint32_t>(p) * static_cast<uint32_t>(n - 1) - static_cast<uint32_t>(p) * static_cast<uint32_t>(p - 1) / 2;
+}
+
+// Minimum over the warp of (score, position), smaller positions first among equal scores; a thread without a weight left
+// has (INFINITY, 0x7fffffff).  On the order-preserving integer images: three 32-bit reductions.
+struct ExBest { uint32_t hi, lo; int pos; };
+__device__ __forceinline__ ExBest ex_key(double score, int pos) {
+    const long long b = __double_as_longlong(score);
+    const unsigned long long k = static_cast<unsigned long long>(b) ^ (b < 0 ? ~0ull : 0x8000000000000000ull);
+    return {static_cast<uint32_t>(k >> 32), static_cast<uint32_t>(k), pos};
+}
+__device__ __forceinline__ ExBest ex_warp_min(ExBest x) {
+    ExBest r;
+    r.hi = __reduce_min_sync(0xffffffffu, x.hi);
+    r.lo = __reduce_min_sync(0xffffffffu, x.hi == r.hi ? x.lo : 0xffffffffu);
+    r.pos = __reduce_min_sync(0xffffffffu, x.hi == r.hi && x.lo == r.lo ? x.pos : 0x7fffffff);
+    return r;
+}
+
+// PER: weights per thread (4 up to c = 1024: the column stays in registers; else EX_MAX_PER).
+template <typename T, bool AFFINE, int PER>
 __global__ void __launch_bounds__(EX_THREADS, 2) exact_row_kernel(ExactArgs A) {
+    constexpr int UN = PER <= 4 ? PER : 4;
     extern __shared__ __align__(16) unsigned char ex_smem[];
-    const int c = A.c, nb = A.nb, K = A.K;
-    double* w = reinterpret_cast<double*>(ex_smem);          // c: the row, error-compensated as it goes
+    const int c = A.c, K = A.K;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double* w = reinterpret_cast<double*>(ex_smem);          // c: the row, error-compensated as it goes (by position)
     double* d = w + c;                                       // c: diagonal of the current inverse
-    double* V = d + c;                                       // nb x c: the columns taken out by the steps of the current batch
-    double* rpiv = V + static_cast<size_t>(nb) * c;          // nb: reciprocals of their pivots
-    double* arow = rpiv + EX_MAX_NB;                         // EX_WARPS x 4 x nb: row coefficients of the batch update
-    double* gpts = arow + EX_WARPS * 4 * EX_MAX_NB;          // 16
-    double* red_s = gpts + 16;                               // 2 x EX_WARPS (alternating between steps)
-    int* red_i = reinterpret_cast<int*>(red_s + 2 * EX_WARPS);      // 2 x EX_WARPS
-    int* rows = red_i + 2 * EX_WARPS;                        // c: rows still to do, ascending (for the batch update)
-    unsigned char* todo = reinterpret_cast<unsigned char*>(rows + c);      // c
-    __shared__ double sh_dii[2];
+    double* V = d + c;                                       // A.vcap: the columns taken out in the current batch, vs apart
+    double* rpiv = V + A.vcap;                               // EX_MAX_NB: reciprocals of their pivots
+    double* gpts = rpiv + EX_MAX_NB;                         // 16, and the 15 midpoints between them
+    double* mids = gpts + 16;
+    double* coef = mids + 16 + warp * EX_MAX_NB;             // a step's  -v_m[i] / pivot_m, by every warp for itself
+    uint16_t* old = reinterpret_cast<uint16_t*>(mids + 16);  // c, in the same place: position before the compaction
+    uint16_t* id = old + ex_names(c);                        // c: the weight at a position, with EX_DONE once it is quantised
+    __shared__ ExBest red[2][EX_WARPS];
+    __shared__ double red_q[2][EX_WARPS];
+    __shared__ int red_c[2][EX_WARPS];
     __shared__ int sh_cnt[EX_WARPS];
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    double* Hi = A.slots + static_cast<size_t>(blockIdx.x) * A.slot_stride;
+    double* slot = A.slots + static_cast<size_t>(blockIdx.x) * A.slot_stride;
+    double* half[2] = {slot, slot + static_cast<size_t>(c) * (c - 1) / 2};
+    // columns of a batch for n weights: what the space holds, whole steps of the MMA where it holds two or more
+    auto batch = [&](int n) {
+        const int most = min(EX_MAX_NB, A.vcap / ex_pitch(n));
+        return most >= 8 ? most & ~3 : most;
+    };
 
     for (int64_t row = blockIdx.x; row < A.r; row += gridDim.x) {
         const T* wp = static_cast<const T*>(A.W) + row * A.ldw;
         for (int j = tid; j < c; j += EX_THREADS) {
             w[j] = ex_load<T>(wp + j);
             d[j] = A.Hinv0[static_cast<size_t>(j) * c + j];
-            todo[j] = 1;
+            id[j] = static_cast<uint16_t>(j);
         }
-        if (!AFFINE && tid < K) gpts[tid] = static_cast<double>(A.grid[row * K + tid]);
-        {   // this row's own copy of the inverse (only its upper triangle is kept up to date below)
-            const double2* src = reinterpret_cast<const double2*>(A.Hinv0);
-            double2* dst = reinterpret_cast<double2*>(Hi);
-            const size_t n2 = static_cast<size_t>(c) * c / 2;
-            for (size_t k = tid; k < n2; k += EX_THREADS) dst[k] = src[k];
-            if ((static_cast<size_t>(c) * c & 1) && tid == 0) Hi[static_cast<size_t>(c) * c - 1] = A.Hinv0[static_cast<size_t>(c) * c - 1];
+        if (!AFFINE && tid < K) {
+            gpts[tid] = static_cast<double>(A.grid[row * K + tid]);
+            if (tid + 1 < K) mids[tid] = 0.5 * (gpts[tid] + static_cast<double>(A.grid[row * K + tid + 1]));
         }
         __syncthreads();
+        const bool ascending = __syncthreads_and(AFFINE || tid + 2 >= K || mids[tid] <= mids[tid + 1]) != 0;
 
-        double loss = 0.0;          // kept by every thread alike
-        int kb = 0;
+        auto quant = [&](double x, int weight, int& code, double& q) {
+            double S = 1.0, Z = 0.0;
+            if (AFFINE) {
+                const int64_t gi = row * A.n_groups + weight / A.group;
+                S = static_cast<double>(A.scale[gi]);
+                Z = static_cast<double>(A.zero[gi]);
+            }
+            ex_quant<AFFINE>(x, gpts, mids, ascending, K, S, Z, code, q);
+        };
+
+        int n = c;                                  // weights the current batch started with
+        int vs = ex_pitch(n), nb = batch(n), kb = 0;
+        const double* M = A.Hinv0;                  // their matrix: U^T U (square) in the first batch, a packed triangle later
+        bool square = true;
+        int to = 0;                                 // half of the slot that the next update writes
+        double loss = 0.0;                          // kept by the first warp
+        // a thread's best weight: loss error (q - w)^2 / (2 Hinv_ii), position, grid point and code.  j ascends within a thread:
+        // first minimum.  A thread whose scores are all infinite or NaN offers its first weight, behind every finite score of
+        // the others.
+        double best = INFINITY, bq = 0.0;
+        int bp = 0x7fffffff, bc = 0;
+        auto offer = [&](int j, int weight, double wj, double dj) {
+            int code;
+            double q;
+            quant(wj, weight, code, q);
+            const double e = q - wj;
+            const double sc = __ddiv_rn(__dmul_rn(e, e), 2.0 * dj);
+            if (sc < best || bp == 0x7fffffff) { bp = j; bq = q; bc = code; }
+            best = sc < best ? sc : best;
+        };
+        for (int j = tid; j < n; j += EX_THREADS) offer(j, j, w[j], d[j]);
         for (int step = 0; step < c; ++step) {
             const int par = step & 1;
-            // (a) the weight with the least loss error (q - w)^2 / (2 Hinv_ii) among those still to do
-            double best = INFINITY;
-            int bi = 0x7fffffff;
-            for (int j = tid; j < c; j += EX_THREADS) {
-                if (!todo[j]) continue;
-                double S = 1.0, Z = 0.0;
-                if (AFFINE) {
-                    const int64_t gi = row * A.n_groups + j / A.group;
-                    S = static_cast<double>(A.scale[gi]);
-                    Z = static_cast<double>(A.zero[gi]);
-                }
-                int code;
-                double q;
-                ex_quant<AFFINE>(w[j], gpts, K, S, Z, code, q);
-                const double e = q - w[j];
-                const double sc = __ddiv_rn(__dmul_rn(e, e), 2.0 * d[j]);
-                if (sc < best) { best = sc; bi = j; }          // j ascends within a thread: first minimum
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-            }
-            if (lane == 0) { red_s[par * EX_WARPS + warp] = best; red_i[par * EX_WARPS + warp] = bi; }
+            // (a) the weight with the least loss error among those still to do
+            const ExBest mine = ex_warp_min(ex_key(best, bp));
+            if (lane == 0) red[par][warp] = mine;
+            if (bp == mine.pos) { red_q[par][warp] = bq; red_c[par][warp] = bc; }       // one lane: positions have one owner
             __syncthreads();
-            best = red_s[par * EX_WARPS];
-            bi = red_i[par * EX_WARPS];
+            const ExBest theirs = red[par][lane & (EX_WARPS - 1)];
+            const int i = ex_warp_min(theirs).pos;
+            const int from = __ffs(__ballot_sync(0xffffffffu, theirs.pos == i)) - 1;
+            const double qi = red_q[par][from];
+            const int code_i = red_c[par][from];
+            // (b) column i of the current inverse: the stored matrix as of the start of the batch, minus the
+            //     batch's downdates  sum_m v_m[j] v_m[i] / pivot_m, which are summed while the column is on its way
+            const uint32_t row_i = square ? static_cast<uint32_t>(i) * c : ex_row(i, n);
+            double vj[PER];
+#pragma unroll UN
+            for (int t = 0; t < PER; ++t) {
+                const int j = tid + t * EX_THREADS;
+                if (j >= n) break;
+                vj[t] = 0.0;
+                if (id[j] < EX_DONE) vj[t] = (square || j >= i) ? M[row_i + j] : M[ex_row(j, n) + i];      // U^T U is symmetric to the bit
+            }
+            const double dii = d[i], wi = w[i], rd = 1.0 / dii;
+            if (lane < kb) coef[lane] = -(V[lane * vs + i] * rpiv[lane]);
+            __syncwarp();
+            const double err = wi - qi;
+            if (warp == 0) loss += __ddiv_rn(__dmul_rn(err, err), 2.0 * dii);
+            best = INFINITY;
+            bp = 0x7fffffff;
+            double acc[UN];
+            if (PER <= 4) {
 #pragma unroll
-            for (int x = 1; x < EX_WARPS; ++x) {
-                const double ob = red_s[par * EX_WARPS + x];
-                const int oi = red_i[par * EX_WARPS + x];
-                if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-            }
-            if (bi == 0x7fffffff) {                             // every score was NaN: take the first weight left
-                for (int j = 0; j < c; ++j) if (todo[j]) { bi = j; break; }
-            }
-            const int i = bi;
-            // its grid point (every thread computes it: cheaper than a broadcast)
-            double qi;
-            int code_i;
-            {
-                double S = 1.0, Z = 0.0;
-                if (AFFINE) {
-                    const int64_t gi = row * A.n_groups + i / A.group;
-                    S = static_cast<double>(A.scale[gi]);
-                    Z = static_cast<double>(A.zero[gi]);
-                }
-                ex_quant<AFFINE>(w[i], gpts, K, S, Z, code_i, qi);
-            }
-            const double err = w[i] - qi;
-            // (b) column i of the current inverse: the stored upper triangle as of the start of the batch, minus the
-            //     batch's downdates  sum_m v_m[j] v_m[i] / pivot_m
-            double vj[EX_PER];
+                for (int t = 0; t < UN; ++t) acc[t] = 0.0;
 #pragma unroll 4
-            for (int t = 0; t < EX_PER; ++t) {
-                const int j = tid + t * EX_THREADS;
-                if (j >= c) break;
-                double x = 0.0;
-                if (todo[j]) {
-                    x = j <= i ? Hi[static_cast<size_t>(j) * c + i] : Hi[static_cast<size_t>(i) * c + j];
-                    for (int m = 0; m < kb; ++m)
-                        x = fma(-(V[static_cast<size_t>(m) * c + i] * rpiv[m]), V[static_cast<size_t>(m) * c + j], x);
-                }
-                vj[t] = x;
-                if (j == i) sh_dii[par] = x;
-            }
-            __syncthreads();
-            // (c) quantise weight i, spread its error (Eq. 3), downdate the diagonal (Eq. 9)
-            const double dii = sh_dii[par];
-            loss += __ddiv_rn(__dmul_rn(err, err), 2.0 * dii);
-#pragma unroll 4
-            for (int t = 0; t < EX_PER; ++t) {
-                const int j = tid + t * EX_THREADS;
-                if (j >= c) break;
-                const double x = vj[t];
-                V[static_cast<size_t>(kb) * c + j] = x;
-                if (j == i) {
-                    w[i] = qi;
-                    todo[i] = 0;
-                    rpiv[kb] = 1.0 / dii;
-                    A.codes[row * c + i] = static_cast<uint8_t>(code_i);
-                    if (A.what) {
-                        if (A.what_bf16) static_cast<__nv_bfloat16*>(A.what)[row * A.ldwh + i] = __float2bfloat16_rn(static_cast<float>(qi));
-                        else static_cast<float*>(A.what)[row * A.ldwh + i] = static_cast<float>(qi);
+                for (int m = 0; m < kb; ++m) {
+                    const double cm = coef[m];
+#pragma unroll
+                    for (int t = 0; t < UN; ++t) {
+                        const int j = tid + t * EX_THREADS;
+                        if (j < n) acc[t] = fma(cm, V[m * vs + j], acc[t]);
                     }
-                    if (!(dii > 0.0)) lq_report(A.dstatus, LQ_ERR_NOT_POSITIVE_DEFINITE, row * c + i);
-                } else if (todo[j]) {
-                    w[j] = __dsub_rn(w[j], __dmul_rn(__ddiv_rn(x, dii), err));
-                    d[j] = __dsub_rn(d[j], __ddiv_rn(__dmul_rn(x, x), dii));
                 }
+            }
+            // (c) quantise weight i, spread its error (Eq. 3), downdate the diagonal (Eq. 9), score what is left
+#pragma unroll UN
+            for (int t = 0; t < PER; ++t) {
+                const int j = tid + t * EX_THREADS;
+                if (j >= n) break;
+                const int nj = id[j];
+                double x = 0.0;
+                if (j == i) {
+                    x = dii;
+                    id[i] = static_cast<uint16_t>(nj | EX_DONE);
+                    rpiv[kb] = rd;
+                    A.codes[row * c + nj] = static_cast<uint8_t>(code_i);
+                    if (A.what) {
+                        if (A.what_bf16) static_cast<__nv_bfloat16*>(A.what)[row * A.ldwh + nj] = __float2bfloat16_rn(static_cast<float>(qi));
+                        else static_cast<float*>(A.what)[row * A.ldwh + nj] = static_cast<float>(qi);
+                    }
+                    if (!(dii > 0.0)) lq_report(A.dstatus, LQ_ERR_NOT_POSITIVE_DEFINITE, row * c + nj);
+                } else if (nj < EX_DONE) {
+                    double a = 0.0;
+                    if (PER <= 4) a = acc[t % UN];
+                    else for (int m = 0; m < kb; ++m) a = fma(coef[m], V[m * vs + j], a);
+                    x = vj[t] + a;
+                    const double g = x * rd;
+                    const double wj = __dsub_rn(w[j], __dmul_rn(g, err));
+                    const double dj = __dsub_rn(d[j], __dmul_rn(x, g));
+                    w[j] = wj;
+                    d[j] = dj;
+                    offer(j, nj, wj, dj);
+                }
+                V[kb * vs + j] = x;
             }
             ++kb;
+            // (d) end of a batch: Hinv[j][l] -= sum_m v_m[j] v_m[l] / pivot_m for the weights j <= l still to do, which move up
+            if (kb < nb || step + 1 == c) continue;
             __syncthreads();
-            // (d) end of a batch: Hinv[j][l] -= sum_m v_m[j] v_m[l] / pivot_m for the rows j still to do, l >= j
-            if (kb == nb && step + 1 < c) {
-                // ascending list of the rows still to do
-                const int per = (c + EX_THREADS - 1) / EX_THREADS;
-                const int j_lo = min(tid * per, c), j_hi = min(j_lo + per, c);
+            {   // ascending list of the positions still to do
+                const int per = (n + EX_THREADS - 1) / EX_THREADS;
+                const int j_lo = min(tid * per, n), j_hi = min(j_lo + per, n);
                 int cnt = 0;
-                for (int j = j_lo; j < j_hi; ++j) cnt += todo[j];
+                for (int j = j_lo; j < j_hi; ++j) cnt += id[j] < EX_DONE ? 1 : 0;
                 int incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -226,81 +298,95 @@ __global__ void __launch_bounds__(EX_THREADS, 2) exact_row_kernel(ExactArgs A) {
                 }
                 if (lane == 31) sh_cnt[warp] = incl;
                 __syncthreads();
-                int base = incl - cnt, nr = 0;
-                for (int x = 0; x < EX_WARPS; ++x) {
-                    if (x < warp) base += sh_cnt[x];
-                    nr += sh_cnt[x];
-                }
+                int base = incl - cnt;
+                for (int x = 0; x < warp; ++x) base += sh_cnt[x];
                 for (int j = j_lo; j < j_hi; ++j)
-                    if (todo[j]) rows[base++] = j;
-                __syncthreads();
-                // each warp takes four rows at a time and walks them in strips of 128 columns (four per lane),
-                // starting at the strip that holds the diagonal of the first of them
-                double* aw = arow + (warp * 4) * EX_MAX_NB;
-                for (int p = warp * 4; p < nr; p += EX_WARPS * 4) {
-                    int jr[4];
-                    double* hr[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        jr[q] = rows[min(p + q, nr - 1)];
-                        hr[q] = Hi + static_cast<size_t>(jr[q]) * c;
-                    }
-                    const int live = min(4, nr - p);
-                    if (lane < kb) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) aw[q * EX_MAX_NB + lane] = V[static_cast<size_t>(lane) * c + jr[q]] * rpiv[lane];
-                    }
-                    {   // the first strip of the four rows this warp takes next is asked for now
-                        const int pn = p + EX_WARPS * 4 + (lane >> 3);
-                        if (pn < nr) {
-                            const int jn = rows[pn];
-                            const int ln = (rows[min(p + EX_WARPS * 4, nr - 1)] & ~127) + (lane & 7) * 16;
-                            if (ln < c) asm volatile("prefetch.global.L2 [%0];" ::"l"(Hi + static_cast<size_t>(jn) * c + ln));
-                        }
-                    }
-                    __syncwarp();
-                    for (int l0 = jr[0] & ~127; l0 < c; l0 += 128) {
-                        {   // the strip after the next of the four rows is asked for now (32 lines of 128 bytes, one per lane)
-                            const int ln = l0 + 256 + (lane & 7) * 16;
-                            if (ln < c) asm volatile("prefetch.global.L2 [%0];" ::"l"(hr[lane >> 3] + ln));
-                            if (l0 == (jr[0] & ~127)) {          // and at the start of a group also the next one
-                                const int l1 = l0 + 128 + (lane & 7) * 16;
-                                if (l1 < c) asm volatile("prefetch.global.L2 [%0];" ::"l"(hr[lane >> 3] + l1));
-                            }
-                        }
-                        double x[4][4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                const int l = l0 + lane + 32 * t;
-                                x[q][t] = (l < c && q < live) ? hr[q][l] : 0.0;
-                            }
-                        for (int m = 0; m < kb; ++m) {
-                            const double* vm = V + static_cast<size_t>(m) * c + l0 + lane;
-                            double y[4];
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) y[t] = (l0 + lane + 32 * t < c) ? vm[32 * t] : 0.0;
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const double cq = aw[q * EX_MAX_NB + m];
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) x[q][t] = fma(-cq, y[t], x[q][t]);
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                const int l = l0 + lane + 32 * t;
-                                if (l < c && q < live) hr[q][l] = x[q][t];
-                            }
-                    }
-                    __syncwarp();
-                }
-                kb = 0;
+                    if (id[j] < EX_DONE) old[base++] = static_cast<uint16_t>(j);
                 __syncthreads();
             }
+            const int n2 = n - kb;
+            double* out = half[to];
+            // Each warp takes eight rows at a time and walks them in strips of 64 columns from the diagonal on.  Of the two
+            // 8 x 8 tiles u of 16 columns, entry e of lane (fr, fk) is column fk + 4 u + 8 e of row fr: four lanes then read
+            // and write a whole 32-byte sector.
+            const int fr = lane >> 2, fk = lane & 3;
+            for (int p = warp * 8; p < n2; p += EX_WARPS * 8) {
+                const int pr = p + fr, o = old[min(pr, n2 - 1)];
+                const double* hr = M + (square ? static_cast<uint32_t>(o) * c : ex_row(o, n));
+                double* hw = out + ex_row(pr, n2);
+                double a[EX_MAX_NB / 4];
+#pragma unroll
+                for (int s4 = 0; s4 < EX_MAX_NB / 4; ++s4) {
+                    const int m = 4 * s4 + fk;
+                    a[s4] = m < kb ? -(V[m * vs + o] * rpiv[m]) : 0.0;
+                }
+                // the strips are asked for ahead of their use (a line of 16 columns per lane): two strips ahead along the
+                // rows, and the first two strips of the rows this warp takes next
+                auto ask = [&](const double* base, int l) {
+                    if (l < n2) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + old[l]));
+                };
+                ask(hr, p + 64 + 16 * fk);
+                {
+                    const int pn = pr + EX_WARPS * 8;
+                    if (pn < n2) {
+                        const int on = old[pn];
+                        const double* hn = M + (square ? static_cast<uint32_t>(on) * c : ex_row(on, n));
+                        ask(hn, max(pn, pn - fr + 16 * fk));
+                        ask(hn, pn - fr + 64 + 16 * fk);
+                    }
+                }
+                for (int l0 = p; l0 < n2; l0 += 64) {
+                    ask(hr, l0 + 128 + 16 * fk);
+                    double x[8][2];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int l = l0 + 16 * (u >> 1) + fk + 4 * (u & 1) + 8 * e;
+                            x[u][e] = (l < n2 && l >= pr) ? hr[old[l]] : 0.0;
+                        }
+                    const double* vb[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int l = l0 + 16 * (u >> 1) + (fr >> 1) + 4 * (u & 1) + 8 * (fr & 1);
+                        vb[u] = V + (l < n2 ? old[l] : 0);
+                    }
+#pragma unroll
+                    for (int s4 = 0; s4 < EX_MAX_NB / 4; ++s4) {
+                        if (4 * s4 >= kb) break;
+                        const int m = min(4 * s4 + fk, kb - 1);           // beyond the batch: a is zero, any entry will do
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) ex_dmma(x[u][0], x[u][1], a[s4], vb[u][m * vs]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int l = l0 + 16 * (u >> 1) + fk + 4 * (u & 1) + 8 * e;
+                            if (l < n2 && l >= pr) hw[l] = x[u][e];
+                        }
+                }
+            }
+            // the weights left move up: their values, diagonals and names (a thread reads before any thread writes)
+            for (int j0 = 0; j0 < n2; j0 += EX_THREADS) {
+                const int j = j0 + tid;
+                double wj = 0.0, dj = 0.0;
+                uint16_t ij = 0;
+                if (j < n2) { const int o = old[j]; wj = w[o]; dj = d[o]; ij = id[o]; }
+                __syncthreads();                    // also: every warp is done with V and the matrix
+                if (j < n2) { w[j] = wj; d[j] = dj; id[j] = ij; }
+            }
+            __syncthreads();
+            M = out;
+            square = false;
+            to ^= 1;
+            n = n2;
+            vs = ex_pitch(n);
+            nb = batch(n);
+            kb = 0;
+            best = INFINITY;
+            bp = 0x7fffffff;
+            for (int j = tid; j < n; j += EX_THREADS) offer(j, id[j], w[j], d[j]);
         }
         if (tid == 0) A.loss_rows[row] = loss;
         __syncthreads();
@@ -321,32 +407,34 @@ __global__ void exact_loss_reduce_kernel(const double* __restrict__ rows, int64_
 }
 
 struct ExactPlan {
-    int nb;
+    int vcap;
     int slots;
     size_t smem;
     size_t off_hinv, off_slots, off_loss, total;
 };
 
-size_t exact_smem(int c, int nb) {
-    return static_cast<size_t>(2 + nb) * c * sizeof(double) + (EX_MAX_NB + EX_WARPS * 4 * EX_MAX_NB + 16 + 2 * EX_WARPS) * sizeof(double) +
-           (2 * EX_WARPS + c) * sizeof(int) + static_cast<size_t>(c) + 16;
+size_t exact_smem(int c, int vcap) {
+    return (static_cast<size_t>(2) * c + vcap + EX_MAX_NB + 32) * sizeof(double) + static_cast<size_t>(ex_names(c) + c) * sizeof(uint16_t);
 }
 
-// Batch length: as long as two CTAs still fit on an SM if that leaves at least 8 steps per batch, else one CTA per SM.
+// Two CTAs per SM if that leaves at least 8 columns per batch, else one.  An SM has 228 KB of shared memory, of which each
+// CTA takes 1 KB for the system and 416 bytes for the static arrays above.
 int exact_plan(int64_t r, int64_t c, int sm_count, ExactPlan* P) {
-    if (c > EX_THREADS * EX_PER) return LQ_ERR_UNSUPPORTED;
-    int nb = 0, per_sm = 2;
-    for (int cand = EX_MAX_NB; cand >= 1; --cand)
-        if (exact_smem(static_cast<int>(c), cand) <= 110 * 1024) { nb = cand; break; }
-    if (nb < 8) {
+    if (c > EX_MAX_C) return LQ_ERR_UNSUPPORTED;
+    const int ci = static_cast<int>(c), vs = ex_pitch(ci);
+    auto room = [&](size_t bytes) {
+        const size_t rest = exact_smem(ci, 0);
+        const int64_t most = static_cast<int64_t>(EX_MAX_NB) * vs, have = rest < bytes ? static_cast<int64_t>((bytes - rest) / sizeof(double)) : 0;
+        return static_cast<int>(have < most ? have : most);
+    };
+    int per_sm = 2;
+    P->vcap = room(114 * 1024 - 1440);
+    if (P->vcap < 8 * vs) {
         per_sm = 1;
-        nb = 0;
-        for (int cand = EX_MAX_NB; cand >= 1; --cand)
-            if (exact_smem(static_cast<int>(c), cand) <= 220 * 1024) { nb = cand; break; }
-        if (nb < 1) return LQ_ERR_UNSUPPORTED;
+        P->vcap = room(220 * 1024);
+        if (P->vcap < vs) return LQ_ERR_UNSUPPORTED;
     }
-    P->nb = nb;
-    P->smem = exact_smem(static_cast<int>(c), nb);
+    P->smem = exact_smem(ci, P->vcap);
     const size_t mat = lq_align_up(static_cast<size_t>(c) * c * sizeof(double), 256);
     int64_t slots = static_cast<int64_t>(sm_count) * per_sm;
     if (slots > r) slots = r;
@@ -428,12 +516,17 @@ extern "C" int lq_quantize_exact(lq_handle* h, void* stream, const lq_config* cf
     A.loss_rows = reinterpret_cast<double*>(wsp + P.off_loss);
     A.dstatus = h->dstatus;
     A.slot_stride = lq_align_up(static_cast<size_t>(c) * c * sizeof(double), 256) / sizeof(double);
-    A.r = r; A.c = static_cast<int>(c); A.K = 1 << cfg->bits; A.nb = P.nb;
+    A.r = r; A.c = static_cast<int>(c); A.K = 1 << cfg->bits; A.vcap = P.vcap;
 
+#define LQ_EXACT_LAUNCH_PER(TT, AFF, PER)                                                                                       \
+    do {                                                                                                                      \
+        LQ_CUDA_TRY(cudaFuncSetAttribute(exact_row_kernel<TT, AFF, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024)); \
+        exact_row_kernel<TT, AFF, PER><<<P.slots, EX_THREADS, P.smem, st>>>(A);                                               \
+    } while (0)
 #define LQ_EXACT_LAUNCH(TT, AFF)                                                                                              \
     do {                                                                                                                      \
-        LQ_CUDA_TRY(cudaFuncSetAttribute(exact_row_kernel<TT, AFF>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024)); \
-        exact_row_kernel<TT, AFF><<<P.slots, EX_THREADS, P.smem, st>>>(A);                                                    \
+        if (c <= 4 * EX_THREADS) LQ_EXACT_LAUNCH_PER(TT, AFF, 4);                                                             \
+        else LQ_EXACT_LAUNCH_PER(TT, AFF, EX_MAX_PER);                                                                        \
     } while (0)
     if (w_dtype == LQ_F32) {
         if (affine) LQ_EXACT_LAUNCH(float, true); else LQ_EXACT_LAUNCH(float, false);
@@ -441,6 +534,7 @@ extern "C" int lq_quantize_exact(lq_handle* h, void* stream, const lq_config* cf
         if (affine) LQ_EXACT_LAUNCH(__nv_bfloat16, true); else LQ_EXACT_LAUNCH(__nv_bfloat16, false);
     }
 #undef LQ_EXACT_LAUNCH
+#undef LQ_EXACT_LAUNCH_PER
     LQ_LAUNCH_CHECK();
     if (loss_out) {
         exact_loss_reduce_kernel<<<1, 256, 0, st>>>(A.loss_rows, r, loss_out);

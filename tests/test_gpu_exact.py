@@ -93,6 +93,45 @@ def test_exact_loop_isolated(lq, h, recipe, r, c, n, kw):
     np.testing.assert_allclose(loss, 0.5 * np.einsum("ri,ij,rj->", D, H_d, D), rtol=1e-6)
 
 
+@pytest.mark.parametrize("r,c,grid,bits", [(3, 1, "sorted", 4), (2, 33, "unsorted", 4), (2, 257, "sorted", 2), (2, 448, "affine", 4),
+                                           (1, 1030, "sorted", 3), (1, 1500, "affine", 3)])
+def test_exact_batch_and_compaction_edges(lq, h, r, c, grid, bits):
+    """Batches that end with one weight left, a batch length that grows with each compaction, widths on both sides of the
+    register column (1024) and of two CTAs per SM (about 1300), a table that does not ascend (the midpoint count then is no
+    bisection).  Inputs as well conditioned as the fp64 rounding of either order needs to give the same decisions."""
+    g = torch.Generator().manual_seed(r * c + bits)
+    U = (torch.triu(torch.randn(c, c, generator=g)) * 0.3 / c ** 0.5 + torch.diag(0.5 + torch.rand(c, generator=g))).float()
+    W = torch.randn(r, c, generator=g) * 0.02
+    kw, tab = {}, {}
+    if grid == "affine":
+        kw = dict(scale=torch.full((r, 1), 0.005), zero=torch.full((r, 1), (1 << bits) // 2, dtype=torch.int32))
+    else:
+        t = torch.randn(r, 1 << bits, generator=g) * 0.03
+        kw = dict(grid=torch.sort(t, dim=1).values if grid == "sorted" else t)
+    cfg = lq.Config.make(grid="affine" if grid == "affine" else "nonuniform", bits=bits, group=0, T=40, t=8)
+    ws = torch.empty(lq.lq_quantize_exact_workspace(cfg, r, c), dtype=torch.uint8, device="cuda")
+    codes = torch.full((r, c), 255, dtype=torch.uint8, device="cuda")
+    what = torch.empty((r, c), dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    lq.lq_quantize_exact(h, cfg, W.cuda(), U.cuda(), codes, ws, W_hat=what, loss_out=loss, **{k: v.cuda() for k, v in kw.items()})
+    lq.lq_sync_status(h)
+    Hinv = f64(U).T @ f64(U)
+    codes = codes.cpu().numpy().astype(np.int64)
+    assert codes.max() < (1 << bits)
+    D = f64(W) - f64(what)
+    np.testing.assert_allclose(loss.item(), 0.5 * np.einsum("ri,ij,rj->", D, np.linalg.inv(Hinv), D), rtol=1e-6)
+    if grid == "unsorted":
+        return          # the oracle's table is sorted by contract; the identity above and the range of the codes hold for any
+    if grid == "affine":
+        tab = dict(scale=f64(kw["scale"]), zero=f64(kw["zero"]), group=0)
+    else:
+        tab = dict(grid=f64(kw["grid"]))
+    codes_o, what_o, loss_o = O.quantize_exact(f64(W), Hinv, bits=bits, **tab)
+    np.testing.assert_array_equal(codes, codes_o)
+    np.testing.assert_allclose(f64(what), what_o, rtol=1e-6, atol=1e-9)
+    np.testing.assert_allclose(loss.item(), loss_o, rtol=1e-9)
+
+
 def test_exact_chained(lq, h):
     L = synth.make_layer("c2", 48, 256, 4096, seed=77)
     kw = dict(grid="nonuniform", bits=3, p=4.0, n_iter=20)
