@@ -155,8 +155,8 @@ static inline int64_t lq_ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b
 // 128 x 256 tiles that lie strictly below the diagonal (symmetric results).
 // The tensor core adds into its fp32 accumulator with truncation, so a long K is cut into
 // segments whose partial sums are added to D with round-to-nearest (seg_iters).
-constexpr int LQ_TC_MAX_PASS = 16;
-constexpr int LQ_TC_MAX_LVL = 5;
+constexpr int LQ_TC_MAX_PASS = 21;       // the pairs (s, t) of six digit slices with s + t <= 7
+constexpr int LQ_TC_MAX_LVL = 6;
 struct lq_tc_gemm_args {
     const void* A_all; int64_t a_rows; int64_t lda;   // a_rows = total rows of A_all; bf16, or 8-bit integers with int8_ops
     const void* B_all; int64_t b_rows; int64_t ldb;
@@ -189,6 +189,18 @@ struct lq_tc_gemm_args {
     // sum is stored to D_first (same shape and leading dimension as D) and does not enter the running sum that goes to
     // D.  An exact leading level and the rounded sum of the other levels then come out of one launch.
     float* D_first;
+    // raw_out: the first two levels leave the running sum, as their int32 sums (exact), to D_first and D_second (both
+    // required; shape and leading dimension of D); D gets the rounded, scaled sum of the others.
+    float* D_second;
+    int raw_out;
+    // Operands with a triangle of zeros (levels, one chunk per level): the k-steps that meet only zeros are left out.
+    //   1: row q of B is zero for k < q;  2: row q of B is zero for k > q;  3: row q of A is zero for k < q
+    // (q counts the product's own rows: row offset a_row_off / b_row_off + q)
+    int tri;
+    // hole > 0 (a multiple of 32; hole_at: of 256): columns [hole_at, hole_at + hole) of the product are left out -- neither computed nor
+    // written; N counts the columns that remain, D and the rows of B keep their places
+    int64_t hole_at, hole;
+    int spare_sms;   // SMs that the launch leaves to kernels on other streams (a persistent CTA keeps its SM until the launch ends)
 };
 int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a);
 

@@ -94,8 +94,15 @@ struct KParams {
     int bk_elems;
     uint32_t idesc_pass[LQ_TC_MAX_PASS];
     float lvl_scale[LQ_TC_MAX_LVL];
-    int first_out;            // the first level's sum is stored through the second output map and leaves the running sum
+    int first_out;            // so many leading levels are stored through output maps of their own and leave the running sum
+    int raw_out;              // as int32
+    int tri;                  // see lq_tc_gemm_args::tri
+    int hole_at, hole;        // see lq_tc_gemm_args::hole
 };
+__device__ __forceinline__ int tile_col(const KParams& p, int tn) {       // first column of a tile
+    const int n0 = tn * 256;
+    return n0 + (n0 >= p.hole_at ? p.hole : 0);
+}
 
 // ---------------------------------------------------------------- PTX wrappers ----
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -336,7 +343,17 @@ __device__ __forceinline__ bool next_piece(const KParams& p, long long& u, long 
 
 // Segment s of a tile: how many (pass, k-block) items it has and which they are.
 struct Seg { int len, kit0, pass0, kb0, kbn; };
-__device__ __forceinline__ Seg seg_of(const KParams& p, int k_blocks, int k_iters, int s) {
+// kr: the k-blocks that the tile needs (all of them unless an operand is triangular).
+struct KRange { int lo, n; };
+__device__ __forceinline__ KRange k_range(const KParams& p, int k_blocks, int tm, int tn) {
+    KRange r = {0, k_blocks};
+    if (p.tri == 1) r.lo = tn * BN / p.bk_elems;
+    if (p.tri == 2) r.n = min(k_blocks, (tn + 1) * BN / p.bk_elems);
+    if (p.tri == 3) r.lo = tm * p.tile_m / p.bk_elems;
+    r.n -= r.lo;
+    return r;
+}
+__device__ __forceinline__ Seg seg_of(const KParams& p, int k_blocks, int k_iters, KRange kr, int s) {
     Seg g;
     if (p.n_lvl == 0) {
         g.kit0 = s * p.seg_iters;
@@ -346,8 +363,8 @@ __device__ __forceinline__ Seg seg_of(const KParams& p, int k_blocks, int k_iter
         const int lvl = s / p.n_chunks, ch = s - lvl * p.n_chunks;
         g.kit0 = 0;
         g.pass0 = p.lvl_pass0[lvl];
-        g.kb0 = ch * p.chunk_kb;
-        g.kbn = min(p.chunk_kb, k_blocks - g.kb0);
+        g.kb0 = kr.lo + ch * p.chunk_kb;
+        g.kbn = min(p.chunk_kb, kr.n - ch * p.chunk_kb);
         g.len = p.lvl_npass[lvl] * g.kbn;
     }
     return g;
@@ -364,7 +381,7 @@ template <int CTAS, bool I8>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_d1,
-                  const __grid_constant__ KParams p) {
+                  const __grid_constant__ CUtensorMap map_d2, const __grid_constant__ KParams p) {
     typedef Cfg<CTAS> C;
     constexpr int STAGES = C::STAGES;
     constexpr bool PAIR = CTAS == 2;
@@ -426,9 +443,10 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             int tm, tn;
             tile_coords(p, pc.tile, tm, tn);
             const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM;
-            const int n0 = tn * BN + static_cast<int>(rank) * C::B_ROWS;
+            const int n0 = tile_col(p, tn) + static_cast<int>(rank) * C::B_ROWS;
+            const KRange kr = k_range(p, k_blocks, tm, tn);
             for (int sg = pc.s0; sg < pc.s1 && alive; ++sg) {
-              const Seg g = seg_of(p, k_blocks, k_iters, sg);
+              const Seg g = seg_of(p, k_blocks, k_iters, kr, sg);
               for (int q = 0; q < g.len; ++q) {
                 if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abortp, p, 1)) { alive = false; break; }
                 if (lane == 0) {
@@ -462,8 +480,14 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         long long u = u_begin;
         Piece pc;
         while (alive && next_piece(p, u, u_stride, pc)) {
+            KRange kr = {0, k_blocks};
+            if (I8 && p.tri) {
+                int tm, tn;
+                tile_coords(p, pc.tile, tm, tn);
+                kr = k_range(p, k_blocks, tm, tn);
+            }
             for (int sg = pc.s0; sg < pc.s1 && alive; ++sg, ++it) {
-                const Seg seg = seg_of(p, k_blocks, k_iters, sg);
+                const Seg seg = seg_of(p, k_blocks, k_iters, kr, sg);
                 const int seg_len = seg.len;
                 const uint32_t acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1;
@@ -524,23 +548,24 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         while (alive && next_piece(p, u, u_stride, pc)) {
             int tm, tn;
             tile_coords(p, pc.tile, tm, tn);
-            const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM, n0 = tn * BN;
+            const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM, n0 = tile_col(p, tn);
+            const int n_end = p.N + (tn * BN >= p.hole_at ? p.hole : 0);
             // the running sums of this thread's row go to D: scale -> swizzled slab -> TMA store or reduce-add
-            auto store_tile = [&](const CUtensorMap* md, bool reduce) {
+            auto store_tile = [&](const CUtensorMap* md, bool reduce, bool as_is) {
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     const int col0 = n0 + hf * (BN / 2) + ch * EPI_COLS;
-                    if (col0 < p.N && m0 < p.M) {
+                    if (col0 < n_end && m0 < p.M) {
                         if (leader) bulk_wait_read<0>();          // the slab buffer has been read out
                         group_bar_sync(1 + hf);
                         uint8_t* rowp = my_buf + row * 128u;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             float4 o;
-                            o.x = p.alpha * accr[ch * 32 + 4 * j + 0];
-                            o.y = p.alpha * accr[ch * 32 + 4 * j + 1];
-                            o.z = p.alpha * accr[ch * 32 + 4 * j + 2];
-                            o.w = p.alpha * accr[ch * 32 + 4 * j + 3];
+                            o.x = as_is ? accr[ch * 32 + 4 * j + 0] : p.alpha * accr[ch * 32 + 4 * j + 0];
+                            o.y = as_is ? accr[ch * 32 + 4 * j + 1] : p.alpha * accr[ch * 32 + 4 * j + 1];
+                            o.z = as_is ? accr[ch * 32 + 4 * j + 2] : p.alpha * accr[ch * 32 + 4 * j + 2];
+                            o.w = as_is ? accr[ch * 32 + 4 * j + 3] : p.alpha * accr[ch * 32 + 4 * j + 3];
                             *reinterpret_cast<float4*>(rowp + ((j ^ (row & 7u)) << 4)) = o;
                         }
                         fence_async_smem();
@@ -553,21 +578,27 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     }
                 }
             };
-            const bool first_out = I8 && p.first_out != 0;
+            const int n_out = I8 ? p.first_out : 0;
+            const bool raw = I8 && p.raw_out != 0;
             bool voted_out = false;
             for (int sg = pc.s0; sg < pc.s1; ++sg, ++it) {
                 const uint32_t acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1;
                 if (!mbar_wait(bar_tfull + 8 * acc, acc_phase, abortp, p, 4)) { alive = false; break; }
                 tc_fence_after();
-                const bool fresh = sg == pc.s0 || (first_out && sg == pc.s0 + 1);       // this segment starts the running sum
+                const bool fresh = sg - pc.s0 <= n_out;                 // this segment starts the running sum (n_out > 0: whole tiles only)
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     uint32_t v[32];
                     tmem_ld32(tmem_base + ((q * 32u) << 16) + acc * BN + hf * (BN / 2) + ch * EPI_COLS, v);
                     tmem_wait_ld();
                     if (I8) {
-                        // int32 partial sums (exact) -> fp32, scaled by the level's power of two
+                        // int32 partial sums (exact) -> fp32, scaled by the level's power of two; raw levels keep their bits
+                        if (raw && sg - pc.s0 < n_out) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) accr[ch * 32 + i] = __uint_as_float(v[i]);
+                            continue;
+                        }
                         const float sc = p.lvl_scale[p.n_lvl > 0 ? sg / p.n_chunks : 0];
                         if (fresh) {
 #pragma unroll
@@ -590,18 +621,18 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (mma_cta) mbar_arrive(bar_tempty + 8 * acc);
                     else mbar_arrive_remote(bar_tempty + 8 * acc, 0);
                 }
-                if (first_out && sg == pc.s0) {
-                    // The first level on its own goes out now, while the tensor core works on the next level.  The vote is
+                if (sg - pc.s0 < n_out) {
+                    // A leading level on its own goes out now, while the tensor core works on the next level.  The vote is
                     // the same barrier as the one behind the loop: a warp whose wait ran out above meets this one there.
                     if (group_bar_or(1 + hf, false)) { voted_out = true; break; }
-                    store_tile(&map_d1, false);
+                    store_tile(sg == pc.s0 ? &map_d1 : &map_d2, false, raw);
                 }
             }
             if (voted_out) { alive = false; break; }
             // A wait may have run out in some warps of the group and not in others: the group leaves together, or
             // the warps that went on would wait at the slab barriers below for warps that never come.
             if (group_bar_or(1 + hf, !alive)) { alive = false; break; }
-            store_tile(&map_d, p.accumulate != 0);
+            store_tile(&map_d, p.accumulate != 0, false);
         }
         if (leader) bulk_wait<0>();
     }
@@ -709,23 +740,31 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
     const int ctas_per_tile = pairs > 0 ? 2 : 1;
     const int b_rows_box = BN / ctas_per_tile;
 
-    CUtensorMap map_a, map_b, map_d, map_d1;
+    if (a.hole < 0 || (a.hole > 0 && (a.hole % 32 || a.hole_at % BN || a.tri))) return LQ_ERR_INVALID_ARG;
+    const int64_t n_all = a.N + a.hole;
+    CUtensorMap map_a, map_b, map_d, map_d1, map_d2;
     const bool i8 = a.int8_ops != 0;
     const int bk_elems = i8 ? 2 * BK : BK;                 // a k-step is one 128-byte swizzle row of either type
     const CUtensorMapDataType op_dt = i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const int op_bytes = i8 ? 1 : 2;
     if (!make_map_2d(&map_a, op_dt, op_bytes, a.A_all, a.K, a.a_rows, a.lda, bk_elems, BM) ||
         !make_map_2d(&map_b, op_dt, op_bytes, a.B_all, a.K, a.b_rows, a.ldb, bk_elems, b_rows_box) ||
-        !make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.D, a.N, a.M, a.ldd, EPI_COLS, BM))
+        !make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.D, n_all, a.M, a.ldd, EPI_COLS, BM))
         return LQ_ERR_CUDA;
-    map_d1 = map_d;
+    map_d1 = map_d2 = map_d;
+    const int n_out = a.D_first ? (a.raw_out ? 2 : 1) : 0;
     if (a.D_first) {
-        // the first level's sum on its own: integer operands, at least two levels, one segment per level, nothing added to D
-        if (!i8 || a.n_lvl < 2 || a.accumulate || (reinterpret_cast<uintptr_t>(a.D_first) & 15) ||
-            a.chunk_kb < lq_ceil_div(a.K, bk_elems))
+        // leading levels' sums on their own: integer operands, a level more than that, one segment per level, nothing added to D
+        if (!i8 || a.n_lvl < n_out + 1 || a.accumulate || (reinterpret_cast<uintptr_t>(a.D_first) & 15) ||
+            a.chunk_kb < lq_ceil_div(a.K, bk_elems) || (a.raw_out && (!a.D_second || (reinterpret_cast<uintptr_t>(a.D_second) & 15))))
             return LQ_ERR_INVALID_ARG;
-        if (!make_map_2d(&map_d1, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.D_first, a.N, a.M, a.ldd, EPI_COLS, BM)) return LQ_ERR_CUDA;
+        const CUtensorMapDataType out_dt = a.raw_out ? CU_TENSOR_MAP_DATA_TYPE_INT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+        if (!make_map_2d(&map_d1, out_dt, 4, a.D_first, n_all, a.M, a.ldd, EPI_COLS, BM) ||
+            (a.raw_out && !make_map_2d(&map_d2, out_dt, 4, a.D_second, n_all, a.M, a.ldd, EPI_COLS, BM)))
+            return LQ_ERR_CUDA;
     }
+    if (a.tri && (!i8 || a.n_lvl < 1 || a.chunk_kb < lq_ceil_div(a.K, bk_elems) || a.tri > 3 || (a.tri == 3 ? a.M : a.N) > a.K))
+        return LQ_ERR_INVALID_ARG;
 
     KParams p;
     p.M = static_cast<int>(a.M);
@@ -762,7 +801,11 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         p.idesc_pass[i] = ctas_per_tile == 2 ? Cfg<2>::idesc_i8(a.a_signed[i] != 0, a.b_signed[i] != 0)
                                              : Cfg<1>::idesc_i8(a.a_signed[i] != 0, a.b_signed[i] != 0);
     for (int i = 0; i < LQ_TC_MAX_LVL; ++i) p.lvl_scale[i] = a.lvl_scale[i];
-    p.first_out = a.D_first ? 1 : 0;
+    p.first_out = n_out;
+    p.raw_out = a.raw_out ? 1 : 0;
+    p.tri = a.tri;
+    p.hole_at = a.hole > 0 ? static_cast<int>(a.hole_at) : 0;
+    p.hole = static_cast<int>(a.hole);
     if (p.num_tiles == 0) return LQ_OK;
     {
         const int k_blocks = static_cast<int>(lq_ceil_div(a.K, bk_elems));
@@ -786,7 +829,8 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         }
     }
     // number of K parts: the one that leaves the shortest schedule, ceil(tiles * q / workers) / q
-    const int workers = ctas_per_tile == 2 ? pairs : h->sm_count;
+    int workers = ctas_per_tile == 2 ? pairs : h->sm_count;
+    if (a.spare_sms > 0 && workers > a.spare_sms / ctas_per_tile) workers -= a.spare_sms / ctas_per_tile;
     p.k_parts = 1;
     if (a.accumulate && p.segs_per_tile >= 16) {          // long K only: every unit pays one epilogue
         double best = static_cast<double>(lq_ceil_div(p.num_tiles, workers));
@@ -809,16 +853,16 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        const cudaError_t le = i8 ? cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, true>, map_a, map_b, map_d, map_d1, p)
-                                  : cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, false>, map_a, map_b, map_d, map_d1, p);
+        const cudaError_t le = i8 ? cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, true>, map_a, map_b, map_d, map_d1, map_d2, p)
+                                  : cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, false>, map_a, map_b, map_d, map_d1, map_d2, p);
         if (le != cudaSuccess) {
             cudaGetLastError();
             return LQ_ERR_CUDA;
         }
         lq_launches_total.fetch_add(1, std::memory_order_relaxed);
     } else {
-        if (i8) lq_tc_gemm_kernel<1, true><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, p);
-        else lq_tc_gemm_kernel<1, false><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, p);
+        if (i8) lq_tc_gemm_kernel<1, true><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
+        else lq_tc_gemm_kernel<1, false><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
         LQ_LAUNCH_CHECK();
     }
     return LQ_OK;

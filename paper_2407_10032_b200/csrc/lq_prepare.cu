@@ -381,21 +381,6 @@ __device__ __forceinline__ void digits_of(double x, int e, __nv_bfloat16 (&d)[NS
         w *= 0.00390625;
     }
 }
-// The same number as signed 8-bit integers for the integer tensor-core path: balanced digits in [-128, 127].  With
-// that range the digits after position s can make up anything in [-128/255, 127/255] of position s, so a digit is
-// chosen to leave its remainder in that interval: q = floor(rest + 128/255).  (Unsigned lower digits would be simpler,
-// but their mean of 127 puts a large common component into every lower level, and the fp32 rounding of that level's
-// sum then costs five bits of the result: measured, 1e-7 instead of 4e-8 on U.)
-__device__ __forceinline__ void digits_of(double x, int e, uint8_t (&d)[NSL]) {
-    double rest = scalbn(x, 8 - e);                     // |rest| <= 127 (exp_for8)
-#pragma unroll
-    for (int s = 0; s < NSL; ++s) {
-        double q = s + 1 < NSL ? floor(rest + 128.0 / 255.0) : rint(rest);
-        q = fmin(fmax(q, -128.0), 127.0);
-        d[s] = static_cast<uint8_t>(static_cast<int8_t>(static_cast<int>(q)));
-        rest = (rest - q) * 256.0;
-    }
-}
 // Exponent for the integer digits: the leading digit must not reach 128.
 __device__ __forceinline__ int exp_for8(double mx) {
     if (!(mx > 0.0)) return 0;
@@ -405,9 +390,8 @@ __device__ __forceinline__ int exp_for8(double mx) {
 }
 
 // Rows [0, rows) of the panel buffer (K columns each): exponent and slices.  One CTA per row.
-template <typename D>
 __global__ void __launch_bounds__(256)
-slice_rows_kernel(const double* __restrict__ P, int64_t ldp, int K, int* __restrict__ ex, D* __restrict__ SL,
+slice_rows_kernel(const double* __restrict__ P, int64_t ldp, int K, int* __restrict__ ex, __nv_bfloat16* __restrict__ SL,
                   int64_t slice_rows) {
     __shared__ double red[8];
     const int64_t row = blockIdx.x;
@@ -427,13 +411,13 @@ slice_rows_kernel(const double* __restrict__ P, int64_t ldp, int K, int* __restr
     mx = red[0];
 #pragma unroll
     for (int w = 1; w < 8; ++w) mx = fmax(mx, red[w]);
-    const int e = isfinite(mx) ? (sizeof(D) == 1 ? exp_for8(mx) : exp_for(mx)) : 0;
+    const int e = isfinite(mx) ? exp_for(mx) : 0;
     if (threadIdx.x == 0) LQ_AT(ex + row) = e;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int kx = threadIdx.x + 256 * u;
         if (kx >= K) continue;
-        D d[NSL];
+        __nv_bfloat16 d[NSL];
         digits_of(isfinite(v[u]) ? v[u] : 0.0, e, d);
 #pragma unroll
         for (int s = 0; s < NSL; ++s) LQ_AT(SL + (s * slice_rows + row) * LDP + kx) = d[s];
@@ -442,7 +426,7 @@ slice_rows_kernel(const double* __restrict__ P, int64_t ldp, int K, int* __restr
 
 // Exponents of the columns j >= col0 of the K rows of A that start at row0 (the final rows of U of an outer block).
 __global__ void __launch_bounds__(256)
-col_exp_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K, int64_t col0, int* __restrict__ ex, int int8) {
+col_exp_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K, int64_t col0, int* __restrict__ ex) {
     // 32 columns per CTA, eight threads per column (each takes every eighth row), so that a column's K loads do not queue
     // behind one another in one thread
     __shared__ double part[8][32];
@@ -456,15 +440,14 @@ col_exp_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K, in
     if (ty == 0 && j < cp) {
 #pragma unroll
         for (int q = 1; q < 8; ++q) mx = fmax(mx, part[q][tx]);
-        LQ_AT(ex + j) = isfinite(mx) ? (int8 ? exp_for8(mx) : exp_for(mx)) : 0;
+        LQ_AT(ex + j) = isfinite(mx) ? exp_for(mx) : 0;
     }
 }
 
 // Slices of those columns, transposed: SL[s][j][kx] = digit s of A[row0 + kx][j].  64 x 64 tiles through shared memory.
-template <typename D>
 __global__ void __launch_bounds__(256)
 slice_cols_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K, int64_t col0, const int* __restrict__ ex,
-                  D* __restrict__ SL, int64_t slice_rows) {
+                  __nv_bfloat16* __restrict__ SL, int64_t slice_rows) {
     __shared__ double tile[64][65];
     const int64_t j0 = col0 + (int64_t)blockIdx.x * 64;
     const int k0 = blockIdx.y * 64;
@@ -479,7 +462,7 @@ slice_cols_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K,
         const int64_t j = j0 + b;
         if (j >= cp || k0 + a >= K) continue;
         const double x = tile[a][b];
-        D d[NSL];
+        __nv_bfloat16 d[NSL];
         digits_of(isfinite(x) ? x : 0.0, LQ_AT(ex + j), d);
 #pragma unroll
         for (int s = 0; s < NSL; ++s) LQ_AT(SL + (s * slice_rows + j) * LDP + k0 + a) = d[s];
@@ -487,16 +470,16 @@ slice_cols_kernel(const double* __restrict__ A, int64_t cp, int64_t row0, int K,
 }
 
 // A[row0 + i][col0 + j] -= 2^(ex[row0 + i] + ex[col0 + j]) (Ta[i][col0 + j] + Tb[i][col0 + j]) over nrows x ncols entries;
-// with `upper`, only the 128 x 128 blocks on or above the diagonal.  Two columns per thread.
+// with `upper`, only the 128 x 128 blocks on or above the diagonal; columns [hole0, hole1) are left out.  Two columns per thread.
 __global__ void __launch_bounds__(256)
 apply_kernel(double* __restrict__ A, int64_t cp, const float* __restrict__ Ta, const float* __restrict__ Tb, int64_t ldt,
-             const int* __restrict__ ex, int64_t row0, int64_t nrows, int64_t col0, int64_t ncols, int upper) {
+             const int* __restrict__ ex, int64_t row0, int64_t nrows, int64_t col0, int64_t ncols, int upper, int64_t hole0, int64_t hole1) {
     const int64_t i = blockIdx.y;
     const int64_t row = row0 + i;
     const int er = LQ_AT(ex + row);
     for (int64_t j2 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 2 * j2 < ncols; j2 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t col = col0 + 2 * j2;
-        if (upper && col / NB < row / NB) continue;
+        if ((upper && col / NB < row / NB) || (col >= hole0 && col < hole1)) continue;
         const float2 a = LQ_AT(reinterpret_cast<const float2*>(Ta + i * ldt + col));
         const float2 b = LQ_AT(reinterpret_cast<const float2*>(Tb + i * ldt + col));
         double2* ap = reinterpret_cast<double2*>(A + row * cp + col);
@@ -745,6 +728,184 @@ __global__ void dinv_kernel(const double* __restrict__ part, int64_t c, int n_ch
     LQ_AT(dinv + j) = static_cast<float>(t);
 }
 
+// ------------------------------------------- outer blocks as digit products (wide matrices) ----
+// Inside an outer block only its own 1024 x 1024 diagonal part goes through the steps diag / panel / update; everything else
+// the block's steps do is three products with its inverse factor V, of inner dimension 1024, on the integer tensor cores:
+//   P = A[above][block] V^T,   A[above][block] = -P V,   A[block][right] = V A[block][right]   (final rows of U).
+// Six digits per operand (47 bits below the largest entry), 21 digit products; the two leading levels leave the tensor core as
+// their exact int32 sums T1, T2, the rest as one fp32 sum T3, and x = 2^(ea + eb) (2^-16 T1 + 2^-24 T2 + T3).  One digit more than
+// the far tiles get, because P is not a sum of terms of its own size: entries of V are up to sqrt(cond) times larger.  The
+// columns of A and of V meet at an index t that carries the scale of feature t (A[i][t] ~ s_t, V[q][t] ~ 1 / s_t): both are
+// balanced by a power of two 2^f(t) near sqrt(A[t][t]) before the digits are taken.
+constexpr int NSW = 6;
+
+// Digits of x 2^sh, |x 2^sh| <= 127 256^(NS - 1) (exp_for8), leading digit first: the balanced digits in [-128, 127] of an integer
+// are its bytes after 128 has been added to every byte.  (Unsigned lower digits would be simpler, but their mean of 127 puts a
+// large common component into every lower level, and the fp32 rounding of that level's sum then costs five bits of the
+// result: measured, 1e-7 instead of 4e-8 on U.)
+template <int NS>
+__device__ __forceinline__ void int_digits(double x, int sh, uint32_t (&d)[NS]) {
+    constexpr long long BIAS = NS == 6 ? 0x808080808080ll : 0x8080808080ll;
+    const long long y = __double2ll_rn(scalbn(x, sh)) + BIAS;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) d[s] = static_cast<uint32_t>((y >> (8 * (NS - 1 - s))) & 0xff) ^ 0x80u;
+}
+// Four consecutive entries of a row: their digits, one 32-bit store per slice.
+template <int NS>
+__device__ __forceinline__ void store_digits(const double (&v)[4], int e, uint8_t* dst, int64_t slice_bytes) {
+    uint32_t w[NS] = {};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        uint32_t d[NS];
+        int_digits<NS>(isfinite(v[u]) ? v[u] : 0.0, 8 * NS - e, d);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) w[s] |= d[s] << (8 * u);
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) LQ_AT(reinterpret_cast<uint32_t*>(dst + s * slice_bytes)) = w[s];
+}
+__device__ __forceinline__ double cta_max256(double mx, double* red) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = red[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) mx = fmax(mx, red[w]);
+    return mx;
+}
+
+// f(t) = floor(log2(A[t][t]) / 2) of the block's diagonal, before its steps overwrite it.
+__global__ void shift_kernel(const double* __restrict__ D, int64_t cp, int K, int* __restrict__ f) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= K) return;
+    const double x = LQ_AT(D + t * cp + t);
+    LQ_AT(f + t) = x > 0.0 && isfinite(x) ? ilogb(x) >> 1 : 0;
+}
+
+// Rows src[row][0..K) (fp64, row stride ld), entry t times 2^(sign f(t)): exponent ex[row] and NSW digits.  One CTA per row.
+__global__ void __launch_bounds__(256)
+slice_rows_wide_kernel(const double* __restrict__ src, int64_t ld, int K, const int* __restrict__ f, int sign, int* __restrict__ ex,
+                       uint8_t* __restrict__ SL, int64_t slice_bytes) {
+    __shared__ double red[8];
+    const int64_t row = blockIdx.x;
+    const int t = 4 * threadIdx.x;
+    double v[4] = {0.0, 0.0, 0.0, 0.0}, mx = 0.0;
+    if (t < K) {
+        const double2* p = reinterpret_cast<const double2*>(src + row * ld + t);
+        const double2 a = LQ_AT(p), b = LQ_AT(p + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = scalbn(v[u], sign * LQ_AT(f + t + u));
+            mx = fmax(mx, fabs(v[u]));
+        }
+    }
+    mx = cta_max256(mx, red);
+    const int e = isfinite(mx) ? exp_for8(mx) : 0;
+    if (threadIdx.x == 0) LQ_AT(ex + row) = e;
+    if (t < K) store_digits<NSW>(v, e, SL + row * LDP + t, slice_bytes);
+}
+
+// Columns [col0, col0 + gridDim.x * 32) below col1 of the K rows src[0..K): exponent ex[j - col0] and NS digits of entry t times
+// 2^(-f(t)) (f may be null), transposed: slice row j - col0 holds the column.  32 columns per CTA: their largest entries
+// first, then the digits (the second read comes out of the L2).  1024 threads, because there may be 32 CTAs only: with 256 the
+// digits of 1024 columns took 118 us.
+constexpr int SC_THREADS = 1024;
+template <int NS>
+__global__ void __launch_bounds__(SC_THREADS)
+slice_cols_wide_kernel(const double* __restrict__ src, int64_t ld, int K, int64_t col0, int64_t col1, const int* __restrict__ f,
+                       int* __restrict__ ex, uint8_t* __restrict__ SL, int64_t slice_bytes) {
+    __shared__ double tile[128][33];
+    __shared__ double part[32][33];
+    __shared__ int sh_e[32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t j0 = col0 + blockIdx.x * 32LL, j = j0 + tx;
+    double mx = 0.0;
+    if (j < col1) {
+#pragma unroll 8
+        for (int t = ty; t < K; t += 32) {
+            const double x = LQ_AT(src + t * ld + j);
+            mx = fmax(mx, fabs(f ? scalbn(x, -LQ_AT(f + t)) : x));
+        }
+    }
+    part[ty][tx] = mx;
+    __syncthreads();
+    mx = part[tx][ty];                                   // warp ty: column ty
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (tx == 0) {
+        const int e = isfinite(mx) ? exp_for8(mx) : 0;
+        sh_e[ty] = e;
+        if (j0 + ty < col1) LQ_AT(ex + (j0 + ty - col0)) = e;
+    }
+    for (int t0 = 0; t0 < K; t0 += 128) {                // K is a multiple of 128
+        __syncthreads();
+#pragma unroll
+        for (int a = ty; a < 128; a += 32) {
+            double x = j < col1 ? LQ_AT(src + (t0 + a) * ld + j) : 0.0;
+            if (f) x = scalbn(x, -LQ_AT(f + t0 + a));
+            tile[a][tx] = x;
+        }
+        __syncthreads();
+        const int b = threadIdx.x >> 5, a = (threadIdx.x & 31) * 4;      // column j0 + b, entries t0 + a ..
+        if (j0 + b < col1) {
+            const double v[4] = {tile[a][b], tile[a + 1][b], tile[a + 2][b], tile[a + 3][b]};
+            store_digits<NS>(v, sh_e[b], SL + (j0 + b - col0) * LDP + t0 + a, slice_bytes);
+        }
+    }
+}
+
+__device__ __forceinline__ double wide_sum(int t1, int t2, float t3, int e) {
+    return scalbn(fma(static_cast<double>(t1), 1.0 / 65536.0, fma(static_cast<double>(t2), 1.0 / 16777216.0, static_cast<double>(t3))), e);
+}
+
+// Rows of P out of their three sums (row stride LDP), straight into digits; ex[row] holds the exponent of the row's left operand
+// and becomes that of P.  One CTA per row.
+__global__ void __launch_bounds__(256)
+slice_sums_kernel(const int* __restrict__ T1, const int* __restrict__ T2, const float* __restrict__ T3, int K, int* __restrict__ ex,
+                  const int* __restrict__ eb, uint8_t* __restrict__ SL, int64_t slice_bytes) {
+    __shared__ double red[8];
+    const int64_t row = blockIdx.x;
+    const int t = 4 * threadIdx.x;
+    const int ea = LQ_AT(ex + row);
+    double v[4] = {0.0, 0.0, 0.0, 0.0}, mx = 0.0;
+    if (t < K) {
+        const int4 a = LQ_AT(reinterpret_cast<const int4*>(T1 + row * LDP + t)), b = LQ_AT(reinterpret_cast<const int4*>(T2 + row * LDP + t));
+        const float4 c = LQ_AT(reinterpret_cast<const float4*>(T3 + row * LDP + t));
+        v[0] = wide_sum(a.x, b.x, c.x, ea + LQ_AT(eb + t));
+        v[1] = wide_sum(a.y, b.y, c.y, ea + LQ_AT(eb + t + 1));
+        v[2] = wide_sum(a.z, b.z, c.z, ea + LQ_AT(eb + t + 2));
+        v[3] = wide_sum(a.w, b.w, c.w, ea + LQ_AT(eb + t + 3));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mx = fmax(mx, fabs(v[u]));
+    }
+    mx = cta_max256(mx, red);                         // its barrier also puts every thread's read of ex[row] before the write
+    const int e = isfinite(mx) ? exp_for8(mx) : 0;
+    if (threadIdx.x == 0) LQ_AT(ex + row) = e;
+    if (t < K) store_digits<NSW>(v, e, SL + row * LDP + t, slice_bytes);
+}
+
+// dst[row][j] = sign * the sum of T1, T2, T3 at (row, j); ea by row, eb by column.  cols is a multiple of 128.
+__global__ void __launch_bounds__(256)
+store_sums_kernel(const int* __restrict__ T1, const int* __restrict__ T2, const float* __restrict__ T3, int64_t ldt, int64_t cols, double sign,
+                  const int* __restrict__ ea, const int* __restrict__ eb, double* __restrict__ dst, int64_t ld) {
+    const int64_t row = blockIdx.y;
+    const int e = LQ_AT(ea + row);
+    for (int64_t j = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); j < cols; j += 4 * (int64_t)gridDim.x * blockDim.x) {
+        const int4 a = LQ_AT(reinterpret_cast<const int4*>(T1 + row * ldt + j)), b = LQ_AT(reinterpret_cast<const int4*>(T2 + row * ldt + j));
+        const float4 c = LQ_AT(reinterpret_cast<const float4*>(T3 + row * ldt + j));
+        double2 lo, hi;
+        lo.x = sign * wide_sum(a.x, b.x, c.x, e + LQ_AT(eb + j));
+        lo.y = sign * wide_sum(a.y, b.y, c.y, e + LQ_AT(eb + j + 1));
+        hi.x = sign * wide_sum(a.z, b.z, c.z, e + LQ_AT(eb + j + 2));
+        hi.y = sign * wide_sum(a.w, b.w, c.w, e + LQ_AT(eb + j + 3));
+        double2* out = reinterpret_cast<double2*>(dst + row * ld + j);
+        LQ_AT(out) = lo;
+        LQ_AT(out + 1) = hi;
+    }
+}
+
 // Launches a kernel of the chain so that it may be placed before its predecessor in the stream has ended (the kernel
 // itself waits with chain_wait()).
 template <typename... KArgs, typename... Args>
@@ -781,27 +942,32 @@ PrepLayout prep_layout(int64_t c) {
     return L;
 }
 
+int launch_apply(cudaStream_t st, double* A, int64_t cp, const float* Ta, const float* Tb, const int* ex, int64_t row0, int64_t nrows,
+                 int64_t col0, int64_t ncols, int upper, int64_t hole0 = 0, int64_t hole1 = 0) {
+    const unsigned gx = static_cast<unsigned>(lq_ceil_div(ncols / 2, 256) < 256 ? lq_ceil_div(ncols / 2, 256) : 256);
+    apply_kernel<<<dim3(gx, static_cast<unsigned>(nrows)), 256, 0, st>>>(A, cp, Ta, Tb, cp, ex, row0, nrows, col0, ncols, upper, hole0, hole1);
+    LQ_LAUNCH_CHECK();
+    return LQ_OK;
+}
+
 // The updates that the steps of outer block [o_lo, o_hi] owe to the tiles outside its rows and columns:
 //   A[i][j] -= sum_k P_i^(k) Q_j^(k)    for block rows i < o_lo and block columns j outside the outer block, j >= i,
 // with Q_j^(k) = P_j^(k)^T left of the outer block (the Cholesky part) and the final row k of U right of it (the
 // Gauss-Jordan part).  Both operands go through the digit slices; row bands of at most `band` rows at a time.
-int deferred_update(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_t o_lo, int64_t o_hi, const double* Pob, int* ex,
-                    void* SL, float* Ta, float* Tb, int64_t band) {
+int deferred_update_bf16(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_t o_lo, int64_t o_hi, const double* Pob, int* ex,
+                         void* SL, float* Ta, float* Tb, int64_t band) {
     const int K = static_cast<int>((o_hi - o_lo + 1) * NB);
     const int64_t top = o_lo * NB;                     // rows [0, top) are updated
     const int64_t right0 = (o_hi + 1) * NB;            // columns [right0, cp) on the right of the outer block
     const int64_t n_right = cp - right0;
-    // digits as 8-bit integers for tcgen05 kind::i8 (twice the rate of the bf16 form), or as bf16 values
-    const bool i8 = h->prep_slices_int8 != 0;
-    if (i8) slice_rows_kernel<uint8_t><<<static_cast<unsigned>(top), 256, 0, st>>>(Pob, LDP, K, ex, static_cast<uint8_t*>(SL), cp);
-    else slice_rows_kernel<__nv_bfloat16><<<static_cast<unsigned>(top), 256, 0, st>>>(Pob, LDP, K, ex, static_cast<__nv_bfloat16*>(SL), cp);
+    __nv_bfloat16* sl = static_cast<__nv_bfloat16*>(SL);
+    slice_rows_kernel<<<static_cast<unsigned>(top), 256, 0, st>>>(Pob, LDP, K, ex, sl, cp);
     LQ_LAUNCH_CHECK();
     if (n_right > 0) {
-        col_exp_kernel<<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), 256, 0, st>>>(A, cp, top, K, right0, ex, i8 ? 1 : 0);
+        col_exp_kernel<<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), 256, 0, st>>>(A, cp, top, K, right0, ex);
         LQ_LAUNCH_CHECK();
         dim3 g(static_cast<unsigned>(lq_ceil_div(n_right, 64)), static_cast<unsigned>(lq_ceil_div(K, 64)));
-        if (i8) slice_cols_kernel<uint8_t><<<g, 256, 0, st>>>(A, cp, top, K, right0, ex, static_cast<uint8_t*>(SL), cp);
-        else slice_cols_kernel<__nv_bfloat16><<<g, 256, 0, st>>>(A, cp, top, K, right0, ex, static_cast<__nv_bfloat16*>(SL), cp);
+        slice_cols_kernel<<<g, 256, 0, st>>>(A, cp, top, K, right0, ex, sl, cp);
         LQ_LAUNCH_CHECK();
     }
     // passes: the leading pair alone (exact), then the pairs of levels s + t = NSL + 1 down to 3, least significant first
@@ -813,20 +979,12 @@ int deferred_update(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_
     lead.K = K;
     lead.alpha = 1.0f;
     lead.n_pass = 1;
-    lead.seg_iters = i8 ? 0 : 4;                       // bf16: 256 digit products per partial sum, far below 2^24; integers: the
-                                                       // whole inner dimension in int32, at most 1024 x 2^14 = 2^24, exact in fp32 too
-    lead.int8_ops = i8 ? 1 : 0;
-    lead.a_signed[0] = lead.b_signed[0] = 1;           // all digits are signed
-    lead.lvl_scale[0] = 1.0f / 65536.0f;               // 2^-8 2^-8 (the bf16 digits carry their power of two themselves)
+    lead.seg_iters = 4;                                // 256 digit products per partial sum, far below 2^24
     lq_tc_gemm_args tail = lead;
     tail.seg_iters = 0;
     tail.n_pass = 0;
     tail.n_lvl = 0;
-    // bf16 digits: 128 of the inner dimension per segment, at most 5 x 128 x 2^14 < 2^24 per partial sum, which the fp32
-    // accumulator holds exactly.  Integer digits: the int32 accumulator holds a level's sum over the whole inner
-    // dimension exactly (5 x 1024 x 2^14 < 2^27), so a level is one segment; its conversion to fp32 rounds at 2^-24 of
-    // a level that lies 2^-8 or more below the leading one.
-    tail.chunk_kb = i8 ? 8 : 2;
+    tail.chunk_kb = 2;             // 128 of the inner dimension per segment: 5 x 128 x 2^14 < 2^24 per partial sum, exact in fp32
     int pair_s[LQ_TC_MAX_PASS], pair_t[LQ_TC_MAX_PASS];
     for (int lvl = NSL + 1; lvl >= 3; --lvl) {
         int cnt = 0;
@@ -835,11 +993,9 @@ int deferred_update(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_
             if (tdig < 1 || tdig > NSL) continue;
             pair_s[tail.n_pass] = sdig - 1;
             pair_t[tail.n_pass] = tdig - 1;
-            tail.a_signed[tail.n_pass] = tail.b_signed[tail.n_pass] = 1;
             ++tail.n_pass;
             ++cnt;
         }
-        tail.lvl_scale[tail.n_lvl] = static_cast<float>(ldexp(1.0, -8 * lvl));
         tail.lvl_npass[tail.n_lvl++] = cnt;
     }
     for (int64_t b0 = 0; b0 < top; b0 += band) {
@@ -849,30 +1005,6 @@ int deferred_update(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_
             const int64_t col0 = side == 0 ? b0 : right0;
             const int64_t ncols = side == 0 ? top - b0 : n_right;
             if (ncols <= 0) continue;
-            if (i8) {
-                // integer digits: one launch, the leading pair as its first level with an output of its own
-                lq_tc_gemm_args g = tail;
-                for (int ps = tail.n_pass; ps > 0; --ps) {
-                    g.a_signed[ps] = tail.a_signed[ps - 1]; g.b_signed[ps] = tail.b_signed[ps - 1];
-                    g.a_row_off[ps] = pair_s[ps - 1] * cp + b0;
-                    g.b_row_off[ps] = pair_t[ps - 1] * cp + col0;
-                }
-                g.a_signed[0] = g.b_signed[0] = 1;
-                g.a_row_off[0] = b0;
-                g.b_row_off[0] = col0;
-                g.n_pass = tail.n_pass + 1;
-                for (int l = tail.n_lvl; l > 0; --l) { g.lvl_npass[l] = tail.lvl_npass[l - 1]; g.lvl_scale[l] = tail.lvl_scale[l - 1]; }
-                g.lvl_npass[0] = 1;
-                g.lvl_scale[0] = lead.lvl_scale[0];
-                g.n_lvl = tail.n_lvl + 1;
-                g.D_first = Ta + col0;
-                g.D = Tb + col0;
-                g.M = b1 - b0;
-                g.N = ncols;
-                g.upper_only = side == 0 ? 1 : 0;
-                int rc = lq_tc_gemm(h, st, g);
-                if (rc) return rc;
-            } else
             for (int which = 0; which < 2; ++which) {
                 lq_tc_gemm_args g = which == 0 ? lead : tail;
                 g.D = (which == 0 ? Ta : Tb) + col0;
@@ -887,11 +1019,216 @@ int deferred_update(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_
                 int rc = lq_tc_gemm(h, st, g);
                 if (rc) return rc;
             }
-            const unsigned gx = static_cast<unsigned>(lq_ceil_div(ncols / 2, 256) < 256 ? lq_ceil_div(ncols / 2, 256) : 256);
-            apply_kernel<<<dim3(gx, static_cast<unsigned>(b1 - b0)), 256, 0, st>>>(A, cp, Ta, Tb, cp, ex, b0, b1 - b0, col0, ncols,
-                                                                                 side == 0 ? 1 : 0);
+            int rc = launch_apply(st, A, cp, Ta, Tb, ex, b0, b1 - b0, col0, ncols, side == 0 ? 1 : 0);
+            if (rc) return rc;
+        }
+    }
+    return LQ_OK;
+}
+
+// ------------------------------------------------------------------ the sweep on wide matrices --
+// The products of NS digits per operand, integer digits: levels s + t = 2 .. NS + 1.  The leading level, exact, has an output of
+// its own (raw: the two leading ones, as int32), then the others, least significant first.
+lq_tc_gemm_args digit_product(int ns, bool raw, const uint8_t* Aall, int64_t a_rows, int64_t a_slice, int64_t a0, const uint8_t* Ball,
+                              int64_t b_rows, int64_t b_slice, int64_t b0, int64_t M, int64_t N, int K) {
+    lq_tc_gemm_args g = {};
+    g.A_all = Aall; g.a_rows = a_rows; g.lda = LDP;
+    g.B_all = Ball; g.b_rows = b_rows; g.ldb = LDP;
+    g.M = M; g.N = N; g.K = K;
+    g.alpha = 1.0f;
+    g.int8_ops = 1;
+    g.chunk_kb = LDP / 128;        // a level is one segment: its int32 sums over the whole inner dimension are exact
+    g.raw_out = raw ? 1 : 0;
+    const int lead = raw ? 2 : 1;
+    for (int i = 0; i < ns; ++i) {
+        const int lvl = i < lead ? 2 + i : ns + 1 - (i - lead);
+        int cnt = 0;
+        for (int sd = 1; sd <= ns; ++sd) {
+            const int td = lvl - sd;
+            if (td < 1 || td > ns) continue;
+            g.a_signed[g.n_pass] = g.b_signed[g.n_pass] = 1;
+            g.a_row_off[g.n_pass] = (sd - 1) * a_slice + a0;
+            g.b_row_off[g.n_pass] = (td - 1) * b_slice + b0;
+            ++g.n_pass;
+            ++cnt;
+        }
+        g.lvl_scale[g.n_lvl] = static_cast<float>(ldexp(1.0, -8 * lvl));
+        g.lvl_npass[g.n_lvl++] = cnt;
+    }
+    return g;
+}
+
+// Block columns are taken in outer blocks of 8, last first.  Per outer block:
+//   chain : its diagonal part D (1024 x 1024) through diag / panel / update -- 8 serial steps of a few tiles -> V
+//   bulk  : digits of V, of the columns of A above D and of the rows right of it; P; then first the update of the next outer
+//           block's diagonal part, after which the chain goes on with it; then A[above][block] = -P V, the final rows of U
+//           right of D, and the update of all other tiles:  A[i][j] -= P_i Q_j,  Q = P^T left of the block, U right of it.
+// The chain (0.55 ms per outer block, a dozen SMs for a few microseconds at a time) runs on the high-priority stream beside the
+// bulk of the outer block before it; the persistent products of that time leave it SPARE_SMS SMs.
+constexpr int SPARE_SMS = 16;
+constexpr double CHAIN_SECONDS = 0.7e-3;      // so long the products leave SMs free
+constexpr double DIGIT_OPS_RATE = 2.2e15;     // integer operations per second of those products (2.2 - 2.6 measured)
+
+int wide_sweep(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_t c, char* wsp, const PrepLayout& L) {
+    const bool fork = h->aux != nullptr && h->chain != nullptr;
+    cudaStream_t cs = fork ? h->chain : st, gs = fork ? h->aux : st;
+    const int64_t n_ob = lq_ceil_div(L.nblk, OBB);
+    double* Ql = reinterpret_cast<double*>(wsp + L.q);                         // step products of D: right operand ...
+    double* Pl = reinterpret_cast<double*>(wsp + L.q + L.panel_bytes);         // ... and panel
+    int* fsh = reinterpret_cast<int*>(wsp + L.q + 2 * L.panel_bytes);          // f(t), two outer blocks alternating
+    int* evt = fsh + 2 * LDP;                                                  // exponents of the columns of V
+    uint8_t* SL = reinterpret_cast<uint8_t*>(wsp + L.sl);                      // slice s of row i of the matrix: s cp + i
+    uint8_t* VT = reinterpret_cast<uint8_t*>(wsp + L.pbuf);                    // slices of the columns of V: s 1024 + q
+    const int64_t sl_bytes = cp * LDP, vt_bytes = static_cast<int64_t>(LDP) * LDP;
+    int* ex = reinterpret_cast<int*>(wsp + L.ex);
+    float* Ta = reinterpret_cast<float*>(wsp + L.ta);
+    float* Tb = reinterpret_cast<float*>(wsp + L.tb);
+    const int64_t t_elems = 2 * L.band * cp;                                   // Ta and Tb lie side by side
+    static_assert(NSW <= 2 * NSL, "the slices' space is laid out for NSL slices of 16-bit digits");
+    if (fork) {
+        LQ_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
+        LQ_CUDA_TRY(cudaStreamWaitEvent(cs, h->ev_fork, 0));
+        LQ_CUDA_TRY(cudaStreamWaitEvent(gs, h->ev_fork, 0));
+    }
+    double busy = 0.0;             // estimated time of the products issued since the chain was let go
+    auto product = [&](lq_tc_gemm_args& g) {
+        g.spare_sms = fork && busy < CHAIN_SECONDS ? SPARE_SMS : 0;
+        busy += 2.0 * g.M * g.N * g.K * g.n_pass * (g.upper_only ? 0.5 : 1.0) * (g.tri ? 0.6 : 1.0) / DIGIT_OPS_RATE;
+        return lq_tc_gemm(h, gs, g);
+    };
+    // the far tiles of rows [r0, r0 + nr) x columns [c0, c1) but [hole0, hole1), those below the diagonal left out
+    auto far_tiles = [&](int64_t r0, int64_t nr, int64_t c0, int64_t c1, int64_t hole0, int64_t hole1, int K) {
+        lq_tc_gemm_args g = digit_product(NSL, false, SL, NSW * cp, cp, r0, SL, NSW * cp, cp, c0, nr, c1 - c0 - (hole1 - hole0), K);
+        g.D_first = Ta + c0;
+        g.D = Tb + c0;
+        g.ldd = cp;
+        g.upper_only = c0 == r0 ? 1 : 0;
+        g.hole_at = hole0 - c0;
+        g.hole = hole1 - hole0;
+        int rc = product(g);
+        return rc ? rc : launch_apply(gs, A, cp, Ta, Tb, ex, r0, nr, c0, c1 - c0, g.upper_only, hole0, hole1);
+    };
+    for (int64_t m = n_ob - 1; m >= 0; --m) {
+        const int64_t o_lo = m * OBB, o_hi = (o_lo + OBB < L.nblk ? o_lo + OBB : L.nblk) - 1;
+        const int obw = static_cast<int>(o_hi - o_lo + 1), K = obw * NB;
+        const int64_t top = o_lo * NB, right0 = top + K, n_right = cp - right0;
+        double* D = A + top * cp + top;
+        int* f = fsh + (m & 1) * LDP;
+        // ---- chain
+        if (m < n_ob - 1 && fork) LQ_CUDA_TRY(cudaStreamWaitEvent(cs, h->ev_next, 0));
+        shift_kernel<<<static_cast<unsigned>(lq_ceil_div(K, 256)), 256, 0, cs>>>(D, cp, K, f);
+        LQ_LAUNCH_CHECK();
+        for (int k = obw - 1; k >= 0; --k) {
+            LQ_CUDA_TRY(launch_chained(diag_block_kernel, dim3(1), dim3(DIAG_THREADS), DIAG_SMEM, cs, A, cp, o_lo + k, c, h->dstatus));
+            if (obw == 1) break;
+            LQ_CUDA_TRY(launch_chained(panel_kernel, dim3(static_cast<unsigned>(4 * (obw - 1))), dim3(GEMM_THREADS), GEMM_SMEM, cs, D, cp, k,
+                                       Pl, static_cast<int64_t>(NB), Ql));
+            if (k == 0) break;
+            update_kernel<<<dim3(static_cast<unsigned>(2 * obw), static_cast<unsigned>(k)), GEMM_THREADS, GEMM_SMEM, cs>>>(
+                D, cp, k, 0, 0, 0, Pl, static_cast<int64_t>(NB), Ql);
             LQ_LAUNCH_CHECK();
         }
+        if (fork) {
+            LQ_CUDA_TRY(cudaEventRecord(h->ev_rest, cs));
+            LQ_CUDA_TRY(cudaStreamWaitEvent(gs, h->ev_rest, 0));
+        }
+        // ---- bulk: digits of V and of the columns above it
+        busy = CHAIN_SECONDS;                                  // nothing runs beside these
+        if (top + n_right > 0) {
+            slice_rows_wide_kernel<<<static_cast<unsigned>(K), 256, 0, gs>>>(D, cp, K, f, 1, ex + top, SL + top * LDP, sl_bytes);
+            LQ_LAUNCH_CHECK();
+        }
+        if (top > 0) {
+            slice_rows_wide_kernel<<<static_cast<unsigned>(top), 256, 0, gs>>>(A + top, cp, K, f, -1, ex, SL, sl_bytes);
+            LQ_LAUNCH_CHECK();
+            // P, straight into digits
+            const int64_t most = t_elems / (3 * LDP) / 256 * 256;
+            for (int64_t r0 = 0; r0 < top; r0 += most) {
+                const int64_t nr = top - r0 < most ? top - r0 : most;
+                lq_tc_gemm_args g = digit_product(NSW, true, SL, NSW * cp, cp, r0, SL, NSW * cp, cp, top, nr, K, K);
+                g.D_first = Ta; g.D_second = Ta + nr * LDP; g.D = Ta + 2 * nr * LDP;
+                g.ldd = LDP;
+                g.tri = 1;
+                int rc = product(g);
+                if (rc) return rc;
+                slice_sums_kernel<<<static_cast<unsigned>(nr), 256, 0, gs>>>(
+                    reinterpret_cast<const int*>(g.D_first), reinterpret_cast<const int*>(g.D_second), g.D, K, ex + r0, ex + top,
+                    SL + r0 * LDP, sl_bytes);
+                LQ_LAUNCH_CHECK();
+            }
+            // the next outer block's diagonal part first: the chain goes on with it
+            const int64_t next = top - LDP;
+            int rc = far_tiles(next, LDP, next, top, top, top, K);
+            if (rc) return rc;
+            if (fork) LQ_CUDA_TRY(cudaEventRecord(h->ev_next, gs));
+            busy = 0.0;
+            slice_cols_wide_kernel<NSW><<<static_cast<unsigned>(K / 32), SC_THREADS, 0, gs>>>(A + top * cp, cp, K, top, right0, nullptr, evt, VT,
+                                                                                             vt_bytes);
+            LQ_LAUNCH_CHECK();
+        }
+        if (n_right > 0) {
+            slice_cols_wide_kernel<NSW><<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), SC_THREADS, 0, gs>>>(
+                A + top * cp, cp, K, right0, cp, f, ex + right0, SL + right0 * LDP, sl_bytes);
+            LQ_LAUNCH_CHECK();
+            // final rows of U right of D, and their digits for the far tiles
+            const int64_t most = t_elems / (3 * LDP) / 256 * 256;
+            for (int64_t j0 = 0; j0 < n_right; j0 += most) {
+                const int64_t nc = n_right - j0 < most ? n_right - j0 : most;
+                lq_tc_gemm_args g = digit_product(NSW, true, SL, NSW * cp, cp, top, SL, NSW * cp, cp, right0 + j0, K, nc, K);
+                g.D_first = Ta; g.D_second = Ta + K * nc; g.D = Ta + 2 * K * nc;
+                g.ldd = nc;
+                g.tri = 3;
+                int rc = product(g);
+                if (rc) return rc;
+                const unsigned gx = static_cast<unsigned>(lq_ceil_div(nc, 1024));
+                store_sums_kernel<<<dim3(gx, static_cast<unsigned>(K)), 256, 0, gs>>>(
+                    reinterpret_cast<const int*>(g.D_first), reinterpret_cast<const int*>(g.D_second), g.D, nc, nc, 1.0, ex + top,
+                    ex + right0 + j0, A + top * cp + right0 + j0, cp);
+                LQ_LAUNCH_CHECK();
+            }
+            if (top > 0) {
+                slice_cols_wide_kernel<NSL><<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), SC_THREADS, 0, gs>>>(
+                    A + top * cp, cp, K, right0, cp, nullptr, ex + right0, SL + right0 * LDP, sl_bytes);
+                LQ_LAUNCH_CHECK();
+            }
+        }
+        if (top > 0) {
+            const int64_t most = t_elems / (3 * LDP) / 256 * 256;
+            for (int64_t r0 = 0; r0 < top; r0 += most) {
+                const int64_t nr = top - r0 < most ? top - r0 : most;
+                lq_tc_gemm_args g = digit_product(NSW, true, SL, NSW * cp, cp, r0, VT, NSW * LDP, LDP, 0, nr, K, K);
+                g.D_first = Ta; g.D_second = Ta + nr * LDP; g.D = Ta + 2 * nr * LDP;
+                g.ldd = LDP;
+                g.tri = 2;
+                int rc = product(g);
+                if (rc) return rc;
+                store_sums_kernel<<<dim3(1, static_cast<unsigned>(nr)), 256, 0, gs>>>(
+                    reinterpret_cast<const int*>(g.D_first), reinterpret_cast<const int*>(g.D_second), g.D, LDP, K, -1.0, ex + r0, evt,
+                    A + r0 * cp + top, cp);
+                LQ_LAUNCH_CHECK();
+            }
+            const int64_t left = top - LDP;                    // the rows of the next outer block have their square already
+            for (int64_t r0 = 0; r0 < top;) {
+                // while the chain runs, a band that ends about when it does: the next one gets the whole chip
+                int64_t nr = L.band;
+                if (fork && busy < CHAIN_SECONDS) {
+                    const double per_row = 2.0 * (cp - K - r0) * K * 15 / DIGIT_OPS_RATE;
+                    const int64_t fit = (static_cast<int64_t>((CHAIN_SECONDS - busy) / per_row) + 255) / 256 * 256;
+                    if (fit < 1024) busy = CHAIN_SECONDS;      // too little to be a launch of its own
+                    else if (fit < nr) nr = fit;
+                }
+                if (r0 < left && r0 + nr > left) nr = left - r0;
+                if (r0 + nr > top) nr = top - r0;
+                const int64_t c0 = r0 < left ? r0 : right0;
+                int rc = c0 < cp ? far_tiles(r0, nr, c0, cp, r0 < left ? top : cp, r0 < left ? right0 : cp, K) : static_cast<int>(LQ_OK);
+                if (rc) return rc;
+                r0 += nr;
+            }
+        }
+    }
+    if (fork) {
+        LQ_CUDA_TRY(cudaEventRecord(h->ev_join, gs));          // the last outer block's products followed the chain
+        LQ_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join, 0));
     }
     return LQ_OK;
 }
@@ -958,8 +1295,14 @@ extern "C" int lq_prepare_hinv(lq_handle* h, void* stream, const float* H, int64
     // kernels and the "next" part of its update stay on the caller's stream; the rest of the eager update goes to
     // the auxiliary stream and overlaps step k-1's diagonal and panel kernels.  When the outer block is complete,
     // all other tiles get its steps' updates in one product on the bf16 tensor cores (deferred_update).
+    const bool defer = nblk > OBB && nblk >= h->prep_defer_min_blocks;
+    const bool wide = defer && h->prep_slices_int8 != 0;
+    if (wide) {
+        int rc = wide_sweep(h, st, A, cp, c, wsp, L);
+        if (rc) return rc;
+    }
     cudaStream_t aux = h->aux;
-    const bool fork = aux != nullptr && nblk > 2;
+    const bool fork = !wide && aux != nullptr && nblk > 2;
     // With the fork the sweep leaves the caller's stream: the chain goes to the handle's high-priority stream `cs`, the
     // bulk of the eager updates to the low-priority `aux`; the caller's stream joins again after the last step.
     cudaStream_t cs = fork ? h->chain : st;
@@ -971,12 +1314,11 @@ extern "C" int lq_prepare_hinv(lq_handle* h, void* stream, const float* H, int64
     double* Pob = reinterpret_cast<double*>(wsp + L.pbuf);
     // Small matrices are bound by the serial chain of diagonal blocks, not by the updates: they stay on the FP64 MMA
     // throughout (one outer block as wide as the matrix).
-    const bool defer = nblk > OBB && nblk >= h->prep_defer_min_blocks;
     const int64_t obb = defer ? OBB : nblk;
-    if (defer) LQ_CUDA_TRY(cudaMemsetAsync(wsp + L.sl, 0, static_cast<size_t>(NSL) * cp * LDP * sizeof(__nv_bfloat16), cs));
+    if (defer && !wide) LQ_CUDA_TRY(cudaMemsetAsync(wsp + L.sl, 0, static_cast<size_t>(NSL) * cp * LDP * sizeof(__nv_bfloat16), cs));
     bool rest_pending = false, next2_pending = false;
     const bool deep = fork && !defer && h->mid != nullptr;
-    const int64_t n_ob = lq_ceil_div(nblk, obb);
+    const int64_t n_ob = wide ? 0 : lq_ceil_div(nblk, obb);
     if (deep) {
         // Nothing deferred (o_lo = 0): look-ahead of two steps, and only what the next diagonal block waits for on the chain.
         //   chain (highest priority): diagonal kernel of step k, then crit_kernel: the panel tile of block row k-1 and the
@@ -1083,7 +1425,7 @@ extern "C" int lq_prepare_hinv(lq_handle* h, void* stream, const float* H, int64
         if (o_lo > 0) {
             if (rest_pending) LQ_CUDA_TRY(cudaStreamWaitEvent(cs, h->ev_rest, 0));
             rest_pending = false;
-            int rc = deferred_update(h, cs, A, cp, o_lo, o_hi, Pob, reinterpret_cast<int*>(wsp + L.ex),
+            int rc = deferred_update_bf16(h, cs, A, cp, o_lo, o_hi, Pob, reinterpret_cast<int*>(wsp + L.ex),
                                      wsp + L.sl, reinterpret_cast<float*>(wsp + L.ta),
                                      reinterpret_cast<float*>(wsp + L.tb), L.band);
             if (rc) return rc;
