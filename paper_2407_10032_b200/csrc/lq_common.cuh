@@ -200,6 +200,10 @@ struct lq_tc_gemm_args {
     // hole > 0 (a multiple of 32; hole_at: of 256): columns [hole_at, hole_at + hole) of the product are left out -- neither computed nor
     // written; N counts the columns that remain, D and the rows of B keep their places
     int64_t hole_at, hole;
+    // integer operands: D's entry (i, j) is multiplied by row_scale[i] col_scale[j] on its way out (powers of two; col_scale is
+    // read up to the end of the last tile: N rounded up to 256 entries)
+    const float* row_scale;
+    const float* col_scale;
     int spare_sms;   // SMs that the launch leaves to kernels on other streams (a persistent CTA keeps its SM until the launch ends)
 };
 int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a);

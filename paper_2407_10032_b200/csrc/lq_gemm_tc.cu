@@ -98,6 +98,8 @@ struct KParams {
     int raw_out;              // as int32
     int tri;                  // see lq_tc_gemm_args::tri
     int hole_at, hole;        // see lq_tc_gemm_args::hole
+    const float* row_scale;   // see lq_tc_gemm_args::row_scale
+    const float* col_scale;
 };
 __device__ __forceinline__ int tile_col(const KParams& p, int tn) {       // first column of a tile
     const int n0 = tn * 256;
@@ -376,8 +378,11 @@ __device__ __forceinline__ void seg_item(const Seg& g, int q, int& pass, int& kb
     kb = g.kb0 + kit - ps * g.kbn;
 }
 
-// I8: the instantiation for 8-bit integer operands; the bf16 instantiation carries none of that code.
-template <int CTAS, bool I8>
+// MODE: BF16 operands, 8-bit integer operands whose sums go out by themselves (INT8_SUMS: stage 2), or 8-bit integer operands
+// whose sum is scaled by row and column and added to D (INT8_SCALED: stage 4).  Each carries its own code only: the epilogue
+// holds 128 running sums per thread and spills with every register more (4 % of a launch for the bf16 form).
+enum { BF16 = 0, INT8_SUMS = 1, INT8_SCALED = 2 };
+template <int CTAS, int MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_d1,
@@ -385,6 +390,7 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     typedef Cfg<CTAS> C;
     constexpr int STAGES = C::STAGES;
     constexpr bool PAIR = CTAS == 2;
+    constexpr bool I8 = MODE != BF16, SUMS = MODE == INT8_SUMS, SCALED = MODE == INT8_SCALED;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[3 * MAX_STAGES + 4];
     __shared__ uint32_t tmem_base_slot;
@@ -443,8 +449,8 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             int tm, tn;
             tile_coords(p, pc.tile, tm, tn);
             const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM;
-            const int n0 = tile_col(p, tn) + static_cast<int>(rank) * C::B_ROWS;
-            const KRange kr = k_range(p, k_blocks, tm, tn);
+            const int n0 = (SUMS ? tile_col(p, tn) : tn * BN) + static_cast<int>(rank) * C::B_ROWS;
+            const KRange kr = SUMS ? k_range(p, k_blocks, tm, tn) : KRange{0, k_blocks};
             for (int sg = pc.s0; sg < pc.s1 && alive; ++sg) {
               const Seg g = seg_of(p, k_blocks, k_iters, kr, sg);
               for (int q = 0; q < g.len; ++q) {
@@ -481,7 +487,7 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         Piece pc;
         while (alive && next_piece(p, u, u_stride, pc)) {
             KRange kr = {0, k_blocks};
-            if (I8 && p.tri) {
+            if (SUMS && p.tri) {
                 int tm, tn;
                 tile_coords(p, pc.tile, tm, tn);
                 kr = k_range(p, k_blocks, tm, tn);
@@ -548,10 +554,11 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         while (alive && next_piece(p, u, u_stride, pc)) {
             int tm, tn;
             tile_coords(p, pc.tile, tm, tn);
-            const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM, n0 = tile_col(p, tn);
-            const int n_end = p.N + (tn * BN >= p.hole_at ? p.hole : 0);
+            const int m0 = tm * C::TILE_M + static_cast<int>(rank) * BM, n0 = SUMS ? tile_col(p, tn) : tn * BN;
+            const int n_end = p.N + (SUMS && tn * BN >= p.hole_at ? p.hole : 0);
             // the running sums of this thread's row go to D: scale -> swizzled slab -> TMA store or reduce-add
-            auto store_tile = [&](const CUtensorMap* md, bool reduce, bool as_is) {
+            auto store_tile = [&](const CUtensorMap* md, bool reduce) {
+                const float rs = SCALED && m0 + static_cast<int>(row) < p.M ? p.alpha * __ldg(p.row_scale + m0 + row) : 0.0f;
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     const int col0 = n0 + hf * (BN / 2) + ch * EPI_COLS;
@@ -562,10 +569,18 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             float4 o;
-                            o.x = as_is ? accr[ch * 32 + 4 * j + 0] : p.alpha * accr[ch * 32 + 4 * j + 0];
-                            o.y = as_is ? accr[ch * 32 + 4 * j + 1] : p.alpha * accr[ch * 32 + 4 * j + 1];
-                            o.z = as_is ? accr[ch * 32 + 4 * j + 2] : p.alpha * accr[ch * 32 + 4 * j + 2];
-                            o.w = as_is ? accr[ch * 32 + 4 * j + 3] : p.alpha * accr[ch * 32 + 4 * j + 3];
+                            if (SCALED) {
+                                const float4 f = __ldg(reinterpret_cast<const float4*>(p.col_scale + col0) + j);
+                                o.x = rs * accr[ch * 32 + 4 * j + 0] * f.x;
+                                o.y = rs * accr[ch * 32 + 4 * j + 1] * f.y;
+                                o.z = rs * accr[ch * 32 + 4 * j + 2] * f.z;
+                                o.w = rs * accr[ch * 32 + 4 * j + 3] * f.w;
+                            } else {
+                                o.x = I8 ? accr[ch * 32 + 4 * j + 0] : p.alpha * accr[ch * 32 + 4 * j + 0];
+                                o.y = I8 ? accr[ch * 32 + 4 * j + 1] : p.alpha * accr[ch * 32 + 4 * j + 1];
+                                o.z = I8 ? accr[ch * 32 + 4 * j + 2] : p.alpha * accr[ch * 32 + 4 * j + 2];
+                                o.w = I8 ? accr[ch * 32 + 4 * j + 3] : p.alpha * accr[ch * 32 + 4 * j + 3];
+                            }
                             *reinterpret_cast<float4*>(rowp + ((j ^ (row & 7u)) << 4)) = o;
                         }
                         fence_async_smem();
@@ -578,15 +593,15 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     }
                 }
             };
-            const int n_out = I8 ? p.first_out : 0;
-            const bool raw = I8 && p.raw_out != 0;
+            const int n_out = SUMS ? p.first_out : 0;
+            const bool raw = SUMS && p.raw_out != 0;
             bool voted_out = false;
             for (int sg = pc.s0; sg < pc.s1; ++sg, ++it) {
                 const uint32_t acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1;
                 if (!mbar_wait(bar_tfull + 8 * acc, acc_phase, abortp, p, 4)) { alive = false; break; }
                 tc_fence_after();
-                const bool fresh = sg - pc.s0 <= n_out;                 // this segment starts the running sum (n_out > 0: whole tiles only)
+                const bool fresh = SUMS ? sg - pc.s0 <= n_out : sg == pc.s0;                 // this segment starts the running sum (n_out > 0: whole tiles only)
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     uint32_t v[32];
@@ -594,7 +609,7 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     tmem_wait_ld();
                     if (I8) {
                         // int32 partial sums (exact) -> fp32, scaled by the level's power of two; raw levels keep their bits
-                        if (raw && sg - pc.s0 < n_out) {
+                        if (SUMS && raw && sg - pc.s0 < n_out) {
 #pragma unroll
                             for (int i = 0; i < 32; ++i) accr[ch * 32 + i] = __uint_as_float(v[i]);
                             continue;
@@ -621,18 +636,18 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (mma_cta) mbar_arrive(bar_tempty + 8 * acc);
                     else mbar_arrive_remote(bar_tempty + 8 * acc, 0);
                 }
-                if (sg - pc.s0 < n_out) {
+                if (SUMS && sg - pc.s0 < n_out) {
                     // A leading level on its own goes out now, while the tensor core works on the next level.  The vote is
                     // the same barrier as the one behind the loop: a warp whose wait ran out above meets this one there.
                     if (group_bar_or(1 + hf, false)) { voted_out = true; break; }
-                    store_tile(sg == pc.s0 ? &map_d1 : &map_d2, false, raw);
+                    store_tile(sg == pc.s0 ? &map_d1 : &map_d2, false);
                 }
             }
             if (voted_out) { alive = false; break; }
             // A wait may have run out in some warps of the group and not in others: the group leaves together, or
             // the warps that went on would wait at the slab barriers below for warps that never come.
             if (group_bar_or(1 + hf, !alive)) { alive = false; break; }
-            store_tile(&map_d, p.accumulate != 0, false);
+            store_tile(&map_d, p.accumulate != 0);
         }
         if (leader) bulk_wait<0>();
     }
@@ -693,8 +708,9 @@ int max_pairs(int sm_count) {
     int& cached = cached_per_device[dev];
     if (!once.first()) return cached;
     cached = 0;
-    if (cudaFuncSetAttribute(lq_tc_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess) {
+    if (cudaFuncSetAttribute(lq_tc_gemm_kernel<2, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, INT8_SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, INT8_SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return cached;
     }
@@ -708,7 +724,7 @@ int max_pairs(int sm_count) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, lq_tc_gemm_kernel<2, false>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, lq_tc_gemm_kernel<2, BF16>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return cached;
     }
@@ -732,18 +748,22 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
 
     static lq_once_per_device attr_set;
     if (attr_set.first()) {
-        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
-        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
+        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
+        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, INT8_SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
+        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, INT8_SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
     }
     // The pair form pays off once there are at least a few 256-row tiles; below that one CTA per tile.
     const int pairs = (a.M > BM) ? max_pairs(h->sm_count) : 0;
     const int ctas_per_tile = pairs > 0 ? 2 : 1;
     const int b_rows_box = BN / ctas_per_tile;
 
+    const bool i8 = a.int8_ops != 0;
     if (a.hole < 0 || (a.hole > 0 && (a.hole % 32 || a.hole_at % BN || a.tri))) return LQ_ERR_INVALID_ARG;
+    if ((a.row_scale != nullptr) != (a.col_scale != nullptr) ||
+        (i8 && !a.row_scale && a.alpha != 1.0f) || (a.row_scale && (!i8 || a.D_first || a.tri || a.hole || (reinterpret_cast<uintptr_t>(a.col_scale) & 15))))
+        return LQ_ERR_INVALID_ARG;
     const int64_t n_all = a.N + a.hole;
     CUtensorMap map_a, map_b, map_d, map_d1, map_d2;
-    const bool i8 = a.int8_ops != 0;
     const int bk_elems = i8 ? 2 * BK : BK;                 // a k-step is one 128-byte swizzle row of either type
     const CUtensorMapDataType op_dt = i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const int op_bytes = i8 ? 1 : 2;
@@ -806,6 +826,8 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
     p.tri = a.tri;
     p.hole_at = a.hole > 0 ? static_cast<int>(a.hole_at) : 0;
     p.hole = static_cast<int>(a.hole);
+    p.row_scale = a.row_scale;
+    p.col_scale = a.col_scale;
     if (p.num_tiles == 0) return LQ_OK;
     {
         const int k_blocks = static_cast<int>(lq_ceil_div(a.K, bk_elems));
@@ -853,16 +875,16 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        const cudaError_t le = i8 ? cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, true>, map_a, map_b, map_d, map_d1, map_d2, p)
-                                  : cudaLaunchKernelEx(&cfg, lq_tc_gemm_kernel<2, false>, map_a, map_b, map_d, map_d1, map_d2, p);
+        const auto kernel = !i8 ? lq_tc_gemm_kernel<2, BF16> : a.row_scale ? lq_tc_gemm_kernel<2, INT8_SCALED> : lq_tc_gemm_kernel<2, INT8_SUMS>;
+        const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, map_d, map_d1, map_d2, p);
         if (le != cudaSuccess) {
             cudaGetLastError();
             return LQ_ERR_CUDA;
         }
         lq_launches_total.fetch_add(1, std::memory_order_relaxed);
     } else {
-        if (i8) lq_tc_gemm_kernel<1, true><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
-        else lq_tc_gemm_kernel<1, false><<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
+        const auto kernel = !i8 ? lq_tc_gemm_kernel<1, BF16> : a.row_scale ? lq_tc_gemm_kernel<1, INT8_SCALED> : lq_tc_gemm_kernel<1, INT8_SUMS>;
+        kernel<<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
         LQ_LAUNCH_CHECK();
     }
     return LQ_OK;

@@ -39,6 +39,7 @@
 //              slices as bf16 values on the bf16 path (exact in its fp32 accumulator per 128 of the inner dimension)
 //              remain selectable for tests; the integer path runs the stage 1.2 - 1.5 x faster.
 #include "lq_common.cuh"
+#include "lq_digits.cuh"
 
 namespace {
 
@@ -364,7 +365,8 @@ crit_kernel(double* __restrict__ A, int64_t cp, int k, int phase, double* __rest
 // x = 2^e (d_1 2^-8 + d_2 2^-16 + ... + d_S 2^-8S) + remainder, with integer digits |d_s| <= 128 and e such that
 // |x| 2^-e <= 1/2 for every entry of the row: slice s holds d_s 2^-8s as bf16 (exact).
 constexpr int OBB = 8;                   // block columns per outer block
-constexpr int LDP = OBB * NB;            // row stride of the panel buffer and of the slices
+constexpr int LDP = LQ_DIGIT_LD;         // row stride of the panel buffer and of the slices
+static_assert(LDP == OBB * NB, "an outer block is one row of digits");
 constexpr int NSL = 5;                   // slices
 constexpr int64_t BAND = 8192;           // rows of the deferred region handled per product
 
@@ -381,14 +383,6 @@ __device__ __forceinline__ void digits_of(double x, int e, __nv_bfloat16 (&d)[NS
         w *= 0.00390625;
     }
 }
-// Exponent for the integer digits: the leading digit must not reach 128.
-__device__ __forceinline__ int exp_for8(double mx) {
-    if (!(mx > 0.0)) return 0;
-    int e = ilogb(mx) + 2;                              // mx 2^(8 - e) < 128
-    if (scalbn(mx, 8 - e) > 127.0) ++e;
-    return e;
-}
-
 // Rows [0, rows) of the panel buffer (K columns each): exponent and slices.  One CTA per row.
 __global__ void __launch_bounds__(256)
 slice_rows_kernel(const double* __restrict__ P, int64_t ldp, int K, int* __restrict__ ex, __nv_bfloat16* __restrict__ SL,
@@ -739,42 +733,6 @@ __global__ void dinv_kernel(const double* __restrict__ part, int64_t c, int n_ch
 // balanced by a power of two 2^f(t) near sqrt(A[t][t]) before the digits are taken.
 constexpr int NSW = 6;
 
-// Digits of x 2^sh, |x 2^sh| <= 127 256^(NS - 1) (exp_for8), leading digit first: the balanced digits in [-128, 127] of an integer
-// are its bytes after 128 has been added to every byte.  (Unsigned lower digits would be simpler, but their mean of 127 puts a
-// large common component into every lower level, and the fp32 rounding of that level's sum then costs five bits of the
-// result: measured, 1e-7 instead of 4e-8 on U.)
-template <int NS>
-__device__ __forceinline__ void int_digits(double x, int sh, uint32_t (&d)[NS]) {
-    constexpr long long BIAS = NS == 6 ? 0x808080808080ll : 0x8080808080ll;
-    const long long y = __double2ll_rn(scalbn(x, sh)) + BIAS;
-#pragma unroll
-    for (int s = 0; s < NS; ++s) d[s] = static_cast<uint32_t>((y >> (8 * (NS - 1 - s))) & 0xff) ^ 0x80u;
-}
-// Four consecutive entries of a row: their digits, one 32-bit store per slice.
-template <int NS>
-__device__ __forceinline__ void store_digits(const double (&v)[4], int e, uint8_t* dst, int64_t slice_bytes) {
-    uint32_t w[NS] = {};
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        uint32_t d[NS];
-        int_digits<NS>(isfinite(v[u]) ? v[u] : 0.0, 8 * NS - e, d);
-#pragma unroll
-        for (int s = 0; s < NS; ++s) w[s] |= d[s] << (8 * u);
-    }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) LQ_AT(reinterpret_cast<uint32_t*>(dst + s * slice_bytes)) = w[s];
-}
-__device__ __forceinline__ double cta_max256(double mx, double* red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) mx = fmax(mx, red[w]);
-    return mx;
-}
-
 // f(t) = floor(log2(A[t][t]) / 2) of the block's diagonal, before its steps overwrite it.
 __global__ void shift_kernel(const double* __restrict__ D, int64_t cp, int K, int* __restrict__ f) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -798,62 +756,13 @@ slice_rows_wide_kernel(const double* __restrict__ src, int64_t ld, int K, const 
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             v[u] = scalbn(v[u], sign * LQ_AT(f + t + u));
-            mx = fmax(mx, fabs(v[u]));
+            mx = fmax(mx, digit_mag(v[u]));
         }
     }
     mx = cta_max256(mx, red);
     const int e = isfinite(mx) ? exp_for8(mx) : 0;
     if (threadIdx.x == 0) LQ_AT(ex + row) = e;
     if (t < K) store_digits<NSW>(v, e, SL + row * LDP + t, slice_bytes);
-}
-
-// Columns [col0, col0 + gridDim.x * 32) below col1 of the K rows src[0..K): exponent ex[j - col0] and NS digits of entry t times
-// 2^(-f(t)) (f may be null), transposed: slice row j - col0 holds the column.  32 columns per CTA: their largest entries
-// first, then the digits (the second read comes out of the L2).  1024 threads, because there may be 32 CTAs only: with 256 the
-// digits of 1024 columns took 118 us.
-constexpr int SC_THREADS = 1024;
-template <int NS>
-__global__ void __launch_bounds__(SC_THREADS)
-slice_cols_wide_kernel(const double* __restrict__ src, int64_t ld, int K, int64_t col0, int64_t col1, const int* __restrict__ f,
-                       int* __restrict__ ex, uint8_t* __restrict__ SL, int64_t slice_bytes) {
-    __shared__ double tile[128][33];
-    __shared__ double part[32][33];
-    __shared__ int sh_e[32];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int64_t j0 = col0 + blockIdx.x * 32LL, j = j0 + tx;
-    double mx = 0.0;
-    if (j < col1) {
-#pragma unroll 8
-        for (int t = ty; t < K; t += 32) {
-            const double x = LQ_AT(src + t * ld + j);
-            mx = fmax(mx, fabs(f ? scalbn(x, -LQ_AT(f + t)) : x));
-        }
-    }
-    part[ty][tx] = mx;
-    __syncthreads();
-    mx = part[tx][ty];                                   // warp ty: column ty
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (tx == 0) {
-        const int e = isfinite(mx) ? exp_for8(mx) : 0;
-        sh_e[ty] = e;
-        if (j0 + ty < col1) LQ_AT(ex + (j0 + ty - col0)) = e;
-    }
-    for (int t0 = 0; t0 < K; t0 += 128) {                // K is a multiple of 128
-        __syncthreads();
-#pragma unroll
-        for (int a = ty; a < 128; a += 32) {
-            double x = j < col1 ? LQ_AT(src + (t0 + a) * ld + j) : 0.0;
-            if (f) x = scalbn(x, -LQ_AT(f + t0 + a));
-            tile[a][tx] = x;
-        }
-        __syncthreads();
-        const int b = threadIdx.x >> 5, a = (threadIdx.x & 31) * 4;      // column j0 + b, entries t0 + a ..
-        if (j0 + b < col1) {
-            const double v[4] = {tile[a][b], tile[a + 1][b], tile[a + 2][b], tile[a + 3][b]};
-            store_digits<NS>(v, sh_e[b], SL + (j0 + b - col0) * LDP + t0 + a, slice_bytes);
-        }
-    }
 }
 
 __device__ __forceinline__ double wide_sum(int t1, int t2, float t3, int e) {
@@ -878,7 +787,7 @@ slice_sums_kernel(const int* __restrict__ T1, const int* __restrict__ T2, const 
         v[2] = wide_sum(a.z, b.z, c.z, ea + LQ_AT(eb + t + 2));
         v[3] = wide_sum(a.w, b.w, c.w, ea + LQ_AT(eb + t + 3));
 #pragma unroll
-        for (int u = 0; u < 4; ++u) mx = fmax(mx, fabs(v[u]));
+        for (int u = 0; u < 4; ++u) mx = fmax(mx, digit_mag(v[u]));
     }
     mx = cta_max256(mx, red);                         // its barrier also puts every thread's read of ex[row] before the write
     const int e = isfinite(mx) ? exp_for8(mx) : 0;
@@ -1162,13 +1071,13 @@ int wide_sweep(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_t c, 
             if (rc) return rc;
             if (fork) LQ_CUDA_TRY(cudaEventRecord(h->ev_next, gs));
             busy = 0.0;
-            slice_cols_wide_kernel<NSW><<<static_cast<unsigned>(K / 32), SC_THREADS, 0, gs>>>(A + top * cp, cp, K, top, right0, nullptr, evt, VT,
+            slice_cols_wide_kernel<NSW><<<static_cast<unsigned>(K / 32), SC_THREADS, 0, gs>>>(A + top * cp, cp, K, top, right0, nullptr, evt, nullptr, VT,
                                                                                              vt_bytes);
             LQ_LAUNCH_CHECK();
         }
         if (n_right > 0) {
             slice_cols_wide_kernel<NSW><<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), SC_THREADS, 0, gs>>>(
-                A + top * cp, cp, K, right0, cp, f, ex + right0, SL + right0 * LDP, sl_bytes);
+                A + top * cp, cp, K, right0, cp, f, ex + right0, nullptr, SL + right0 * LDP, sl_bytes);
             LQ_LAUNCH_CHECK();
             // final rows of U right of D, and their digits for the far tiles
             const int64_t most = t_elems / (3 * LDP) / 256 * 256;
@@ -1188,7 +1097,7 @@ int wide_sweep(lq_handle* h, cudaStream_t st, double* A, int64_t cp, int64_t c, 
             }
             if (top > 0) {
                 slice_cols_wide_kernel<NSL><<<static_cast<unsigned>(lq_ceil_div(n_right, 32)), SC_THREADS, 0, gs>>>(
-                    A + top * cp, cp, K, right0, cp, nullptr, ex + right0, SL + right0 * LDP, sl_bytes);
+                    A + top * cp, cp, K, right0, cp, nullptr, ex + right0, nullptr, SL + right0 * LDP, sl_bytes);
                 LQ_LAUNCH_CHECK();
             }
         }

@@ -11,6 +11,7 @@
 #include <math.h>
 
 #include "lq_common.cuh"
+#include "lq_digits.cuh"
 #include "lq_affine_warp.cuh"
 
 namespace {
@@ -63,12 +64,14 @@ __global__ void to_f32_kernel(const T* __restrict__ W, int64_t ldw, int64_t c, f
     }
 }
 
-// UT[s][n][k] = s-th bf16 term of U[k][n]   (three stacked c x ldt matrices).  64 x 64 tiles: 16-byte reads along n,
-// 16-byte writes (eight bf16) along k.
+// UT[s][n][k - o] = s-th bf16 term of U[k][n] for the rows k of column n's own outer block, which starts at o (three stacked
+// c x ldt matrices): the right operand of the products inside an outer block.  64 x 64 tiles: 16-byte reads along n, 16-byte
+// writes (eight bf16) along k.
 __global__ void __launch_bounds__(256)
 split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv_bfloat16* __restrict__ UT, int64_t ldt) {
     __shared__ float tile[64][65];
-    const int64_t k0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
+    const int64_t n0 = (int64_t)blockIdx.x * 64, o = n0 / OB * OB, k0 = o + (int64_t)blockIdx.y * 64;
+    if (k0 > n0) return;                                // below the diagonal: zero, and never read
     const int tid = threadIdx.x;
     const bool vec_in = (ldu % 4 == 0) && ((reinterpret_cast<uintptr_t>(U) & 15) == 0);
     for (int idx = tid; idx < 64 * 16; idx += 256) {
@@ -90,7 +93,7 @@ split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv
     for (int idx = tid; idx < 64 * 8; idx += 256) {
         const int a = idx >> 3, k8 = (idx & 7) * 8;        // output row n0 + a, eight consecutive k
         const int64_t n = n0 + a, k = k0 + k8;
-        if (n >= c || k >= ldt) continue;
+        if (n >= c || k - o >= ldt) continue;
         uint32_t ph[4], pm[4], pl[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -102,10 +105,35 @@ split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv
             pl[e] = static_cast<uint32_t>(__bfloat16_as_ushort(l0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
         }
         // ldt is a multiple of 8 and k a multiple of 8: the eight entries are inside the row and 16-byte aligned
-        LQ_AT(reinterpret_cast<uint4*>(UT + n * ldt + k)) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-        LQ_AT(reinterpret_cast<uint4*>(UT + (c + n) * ldt + k)) = make_uint4(pm[0], pm[1], pm[2], pm[3]);
-        LQ_AT(reinterpret_cast<uint4*>(UT + (2 * c + n) * ldt + k)) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+        LQ_AT(reinterpret_cast<uint4*>(UT + n * ldt + k - o)) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+        LQ_AT(reinterpret_cast<uint4*>(UT + (c + n) * ldt + k - o)) = make_uint4(pm[0], pm[1], pm[2], pm[3]);
+        LQ_AT(reinterpret_cast<uint4*>(UT + (2 * c + n) * ldt + k - o)) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
     }
+}
+
+// Digits of the rows of E (r x OB, as the in-block kernel left it: three bf16 terms whose sum is the fp32 entry), one exponent
+// per row; scale[row] = 2^e, or NaN when the row holds a NaN or an infinity.  One CTA per row.
+template <int NS>
+__global__ void __launch_bounds__(256)
+slice_errors_kernel(const __nv_bfloat16* __restrict__ ES, int64_t r, float* __restrict__ scale, uint8_t* __restrict__ SL, int64_t slice_bytes) {
+    __shared__ double red[8];
+    const int64_t row = blockIdx.x;
+    const int t = 4 * threadIdx.x;
+    double v[4] = {0.0, 0.0, 0.0, 0.0}, mx = 0.0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const uint2 x = LQ_AT(reinterpret_cast<const uint2*>(ES + (s * r + row) * OB + t));
+        v[0] += static_cast<double>(__uint_as_float(x.x << 16));
+        v[1] += static_cast<double>(__uint_as_float(x.x & 0xffff0000u));
+        v[2] += static_cast<double>(__uint_as_float(x.y << 16));
+        v[3] += static_cast<double>(__uint_as_float(x.y & 0xffff0000u));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) mx = fmax(mx, digit_mag(v[u]));
+    mx = cta_max256(mx, red);
+    const int e = isfinite(mx) ? exp_for8(mx) : 0;
+    if (threadIdx.x == 0) LQ_AT(scale + row) = isfinite(mx) ? ldexpf(1.0f, e) : __int_as_float(0x7fc00000);
+    store_digits<NS>(v, e, SL + row * OB + t, slice_bytes);
 }
 
 struct QuantOut {
@@ -428,19 +456,27 @@ __global__ void loss_reduce_kernel(const double* __restrict__ loss_rows, int64_t
     if (threadIdx.x == 0) loss_out[0] = 0.5 * red[0];
 }
 
+constexpr int FAR_SLICES = 4;            // digits per operand of the products beyond an outer block, at most
 struct WsLayout {
-    size_t wc, ut, es, loss, total;
+    size_t wc, ut, es, loss, ud, ed, cscale, rscale, total;
     int64_t ldc, ldt;
 };
 WsLayout ws_layout(int64_t r, int64_t c) {
     WsLayout L;
     L.ldc = lq_ceil_div(c, 4) * 4;
-    L.ldt = lq_ceil_div(c, 8) * 8;
+    L.ldt = c > OB ? OB : lq_ceil_div(c, 8) * 8;
     size_t off = 0;
     L.wc = off; off += lq_align_up(static_cast<size_t>(r) * L.ldc * sizeof(float), 256);
     L.ut = off; off += lq_align_up(static_cast<size_t>(3) * c * L.ldt * sizeof(__nv_bfloat16), 256);
     L.es = off; off += lq_align_up(static_cast<size_t>(3) * r * OB * sizeof(__nv_bfloat16), 256);
     L.loss = off; off += lq_align_up(static_cast<size_t>(r) * sizeof(double), 256);
+    L.ud = L.ed = L.cscale = L.rscale = off;
+    if (c > OB) {                          // the digits and scales of one outer block's errors and of the rows of U beside it
+        L.ud = off; off += lq_align_up(static_cast<size_t>(FAR_SLICES) * c * OB, 256);
+        L.ed = off; off += lq_align_up(static_cast<size_t>(FAR_SLICES) * r * OB, 256);
+        L.cscale = off; off += lq_align_up(static_cast<size_t>(c + 256) * sizeof(float), 256);      // read up to the end of a tile
+        L.rscale = off; off += lq_align_up(static_cast<size_t>(r) * sizeof(float), 256);
+    }
     L.total = off;
     return L;
 }
@@ -505,6 +541,54 @@ bool lazy_group_ok(int64_t g, int64_t c) {
     if (g < B) return g % 4 == 0 && B % g == 0;        // inside a block: refitted by the in-block kernel itself
     if (g % B) return false;
     return (g <= OB && OB % g == 0) || (g % OB == 0);
+}
+
+// The columns beyond the outer block that starts at o0 get the errors of all its columns, W -= E U, as a product of 8-bit
+// digits on tcgen05 kind::i8: NS balanced digits per entry below the largest entry of its row of E / column of U, the digit
+// pairs s + t <= 5, each level summed exactly in int32 and the levels added in fp32, least significant first.  Twice the rate of
+// bf16 at under half the energy per product, which is what counts on the large layers (they run at the power limit).
+// Against 64 bits, in units of the result's norm (r x 1024 x 3072, errors of real column loops on ill-conditioned Hessians):
+//   three bf16 terms, 6 products (what this replaces; the tensor core truncates its fp32 sums)   5.1e-7 .. 7.0e-7
+//   3 digits, 8 products    non-uniform grids 2.8e-7 .. 5.6e-7, affine groups 8.4e-7
+//   4 digits, 10 products   2.6e-8 .. 3.0e-8
+// so affine grids, whose clipped weights leave a few large errors per row, take the fourth digit.
+template <int NS>
+int far_update(lq_handle* h, cudaStream_t st, const WsLayout& L, char* wsp, const float* U, int64_t ldu, int64_t r, int64_t c, int64_t o0) {
+    const int64_t end = o0 + OB;
+    uint8_t* UD = reinterpret_cast<uint8_t*>(wsp + L.ud);
+    uint8_t* ED = reinterpret_cast<uint8_t*>(wsp + L.ed);
+    float* cscale = reinterpret_cast<float*>(wsp + L.cscale);
+    float* rscale = reinterpret_cast<float*>(wsp + L.rscale);
+    slice_errors_kernel<NS><<<static_cast<unsigned>(r), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(wsp + L.es), r, rscale, ED, r * OB);
+    LQ_LAUNCH_CHECK();
+    slice_cols_wide_kernel<NS><<<static_cast<unsigned>(lq_ceil_div(c - end, 32)), SC_THREADS, 0, st>>>(
+        U + o0 * ldu, ldu, static_cast<int>(OB), end, c, nullptr, nullptr, cscale, UD, c * OB);
+    LQ_LAUNCH_CHECK();
+    lq_tc_gemm_args g = {};
+    g.A_all = ED; g.a_rows = NS * r; g.lda = OB;
+    g.B_all = UD; g.b_rows = NS * c; g.ldb = OB;
+    g.D = reinterpret_cast<float*>(wsp + L.wc) + end; g.ldd = L.ldc;
+    g.M = r; g.N = c - end; g.K = OB;
+    g.alpha = -1.0f; g.accumulate = 1;
+    g.int8_ops = 1;
+    g.chunk_kb = OB / 128;
+    for (int lvl = 5; lvl >= 2; --lvl) {
+        int cnt = 0;
+        for (int s = 1; s <= NS; ++s) {
+            const int t = lvl - s;
+            if (t < 1 || t > NS) continue;
+            g.a_signed[g.n_pass] = g.b_signed[g.n_pass] = 1;
+            g.a_row_off[g.n_pass] = (s - 1) * r;
+            g.b_row_off[g.n_pass] = (t - 1) * c;
+            ++g.n_pass;
+            ++cnt;
+        }
+        g.lvl_scale[g.n_lvl] = static_cast<float>(ldexp(1.0, -8 * lvl));
+        g.lvl_npass[g.n_lvl++] = cnt;
+    }
+    g.row_scale = rscale;
+    g.col_scale = cscale;
+    return lq_tc_gemm(h, st, g);
 }
 
 // dinv != nullptr selects the lazy refit: scale / zero are then outputs, filled group by group as the loop goes.
@@ -579,7 +663,7 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
         LQ_LAUNCH_CHECK();
     }
     if (c > B) {
-        dim3 g(static_cast<unsigned>(lq_ceil_div(c, 64)), static_cast<unsigned>(lq_ceil_div(L.ldt, 64)));
+        dim3 g(static_cast<unsigned>(lq_ceil_div(c, 64)), static_cast<unsigned>(lq_ceil_div(L.ldt, 64)));      // the blocks on the diagonal
         split_transpose_kernel<<<g, 256, 0, st>>>(U, ldu, c, UT, L.ldt);
         LQ_LAUNCH_CHECK();
     }
@@ -642,7 +726,7 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
         if (near > 0) {
             lq_tc_gemm_args g = {};
             g.A_all = ES + (i0 - o0); g.a_rows = 3 * r; g.lda = OB;
-            g.B_all = UT + (i0 + B) * L.ldt + i0; g.b_rows = 3 * c - (i0 + B); g.ldb = L.ldt;
+            g.B_all = UT + (i0 + B) * L.ldt + (i0 - o0); g.b_rows = 3 * c - (i0 + B); g.ldb = L.ldt;
             g.D = Wc + (i0 + B); g.ldd = L.ldc;
             g.M = r; g.N = near; g.K = B;
             g.n_pass = 6;
@@ -652,16 +736,7 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
             if (rc) return rc;
         }
         if (i0 + B >= ob_end && ob_end < c) {
-            lq_tc_gemm_args g = {};
-            g.A_all = ES; g.a_rows = 3 * r; g.lda = OB;
-            g.B_all = UT + ob_end * L.ldt + o0; g.b_rows = 3 * c - ob_end; g.ldb = L.ldt;
-            g.D = Wc + ob_end; g.ldd = L.ldc;
-            g.M = r; g.N = c - ob_end; g.K = ob_end - o0;
-            g.n_pass = 6;
-            for (int i = 0; i < 6; ++i) { g.a_row_off[i] = ao[i]; g.b_row_off[i] = bo[i]; }
-            g.alpha = -1.0f; g.accumulate = 1; g.upper_only = 0;
-            g.seg_iters = 12;          // partial sums leave the tensor core's truncating accumulator every 128 columns
-            rc = lq_tc_gemm(h, st, g);
+            rc = affine ? far_update<4>(h, st, L, wsp, U, ldu, r, c, o0) : far_update<3>(h, st, L, wsp, U, ldu, r, c, o0);
             if (rc) return rc;
         }
     }
