@@ -41,6 +41,36 @@ __device__ __forceinline__ void store_digits(const double (&v)[4], int e, uint8_
 #pragma unroll
     for (int s = 0; s < NS; ++s) LQ_AT(reinterpret_cast<uint32_t*>(dst + s * slice_bytes)) = w[s];
 }
+// The same for fp32 entries and up to four digits, in 32-bit arithmetic: scaling by a power of two is exact and
+// |x 2^(8 NS - e)| <= 127 256^(NS - 1) < 2^31.  (Through fp64 the slices of one outer block of stage 4 took 40 us per 8000 columns.)
+__device__ __forceinline__ int exp_for8(float mx) {
+    if (!(mx > 0.0f)) return 0;
+    int e = ilogbf(mx) + 2;
+    if (scalbnf(mx, 8 - e) > 127.0f) ++e;
+    return e;
+}
+template <int NS>
+__device__ __forceinline__ void store_digits(const float (&v)[4], int e, uint8_t* dst, int64_t slice_bytes) {
+    static_assert(NS <= 4, "32-bit digits");
+    uint32_t y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int x = isfinite(v[u]) ? __float2int_rn(scalbnf(v[u], 8 * NS - e)) : 0;
+        y[u] = (static_cast<uint32_t>(x) + (0x80808080u >> (32 - 8 * NS))) ^ (0x80808080u >> (32 - 8 * NS));
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const int b = 8 * (NS - 1 - s);
+        const uint32_t w = ((y[0] >> b) & 0xffu) | ((y[1] >> b) & 0xffu) << 8 | ((y[2] >> b) & 0xffu) << 16 | ((y[3] >> b) & 0xffu) << 24;
+        LQ_AT(reinterpret_cast<uint32_t*>(dst + s * slice_bytes)) = w;
+    }
+}
+__device__ __forceinline__ float digit_mag(float x) { return isfinite(x) ? fabsf(x) : INFINITY; }
+__device__ __forceinline__ float digit_shift(float x, int n) { return scalbnf(x, n); }
+__device__ __forceinline__ double digit_shift(double x, int n) { return scalbn(x, n); }
+__device__ __forceinline__ float digit_max(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double digit_max(double a, double b) { return fmax(a, b); }
+
 // Magnitude for the choice of an exponent: a NaN must not hide behind fmax.
 __device__ __forceinline__ double digit_mag(double x) { return isfinite(x) ? fabs(x) : INFINITY; }
 __device__ __forceinline__ double cta_max256(double mx, double* red) {
@@ -63,24 +93,24 @@ template <int NS, typename T>
 __global__ void __launch_bounds__(SC_THREADS)
 slice_cols_wide_kernel(const T* __restrict__ src, int64_t ld, int K, int64_t col0, int64_t col1, const int* __restrict__ f,
                        int* __restrict__ ex, float* __restrict__ scale, uint8_t* __restrict__ SL, int64_t slice_bytes) {
-    __shared__ double tile[128][33];
-    __shared__ double part[32][33];
+    __shared__ T tile[128][33];
+    __shared__ T part[32][33];
     __shared__ int sh_e[32];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int64_t j0 = col0 + blockIdx.x * 32LL, j = j0 + tx;
-    double mx = 0.0;
+    T mx = T(0);
     if (j < col1) {
 #pragma unroll 8
         for (int t = ty; t < K; t += 32) {
-            const double x = static_cast<double>(LQ_AT(src + t * ld + j));
-            mx = fmax(mx, digit_mag(f ? scalbn(x, -LQ_AT(f + t)) : x));
+            const T x = LQ_AT(src + t * ld + j);
+            mx = digit_max(mx, digit_mag(f ? digit_shift(x, -LQ_AT(f + t)) : x));
         }
     }
     part[ty][tx] = mx;
     __syncthreads();
     mx = part[tx][ty];                                   // warp ty: column ty
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int o = 16; o > 0; o >>= 1) mx = digit_max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (tx == 0) {
         const int e = isfinite(mx) ? exp_for8(mx) : 0;
         sh_e[ty] = e;
@@ -91,14 +121,14 @@ slice_cols_wide_kernel(const T* __restrict__ src, int64_t ld, int K, int64_t col
         __syncthreads();
 #pragma unroll
         for (int a = ty; a < 128; a += 32) {
-            double x = j < col1 ? static_cast<double>(LQ_AT(src + (t0 + a) * ld + j)) : 0.0;
-            if (f) x = scalbn(x, -LQ_AT(f + t0 + a));
+            T x = j < col1 ? LQ_AT(src + (t0 + a) * ld + j) : T(0);
+            if (f) x = digit_shift(x, -LQ_AT(f + t0 + a));
             tile[a][tx] = x;
         }
         __syncthreads();
         const int b = threadIdx.x >> 5, a = (threadIdx.x & 31) * 4;      // column j0 + b, entries t0 + a ..
         if (j0 + b < col1) {
-            const double v[4] = {tile[a][b], tile[a + 1][b], tile[a + 2][b], tile[a + 3][b]};
+            const T v[4] = {tile[a][b], tile[a + 1][b], tile[a + 2][b], tile[a + 3][b]};
             store_digits<NS>(v, sh_e[b], SL + (j0 + b - col0) * LQ_DIGIT_LD + t0 + a, slice_bytes);
         }
     }

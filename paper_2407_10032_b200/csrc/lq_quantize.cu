@@ -112,28 +112,33 @@ split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv
 }
 
 // Digits of the rows of E (r x OB, as the in-block kernel left it: three bf16 terms whose sum is the fp32 entry), one exponent
-// per row; scale[row] = 2^e, or NaN when the row holds a NaN or an infinity.  One CTA per row.
+// per row; scale[row] = 2^e, or NaN when the row holds a NaN or an infinity.  One warp per row.
 template <int NS>
 __global__ void __launch_bounds__(256)
 slice_errors_kernel(const __nv_bfloat16* __restrict__ ES, int64_t r, float* __restrict__ scale, uint8_t* __restrict__ SL, int64_t slice_bytes) {
-    __shared__ double red[8];
-    const int64_t row = blockIdx.x;
-    const int t = 4 * threadIdx.x;
-    double v[4] = {0.0, 0.0, 0.0, 0.0}, mx = 0.0;
+    const int lane = threadIdx.x & 31;
+    const int64_t row = blockIdx.x * 8LL + (threadIdx.x >> 5);
+    if (row >= r) return;
+    float v[OB / 128][4], mx = 0.0f;
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const uint2 x = LQ_AT(reinterpret_cast<const uint2*>(ES + (s * r + row) * OB + t));
-        v[0] += static_cast<double>(__uint_as_float(x.x << 16));
-        v[1] += static_cast<double>(__uint_as_float(x.x & 0xffff0000u));
-        v[2] += static_cast<double>(__uint_as_float(x.y << 16));
-        v[3] += static_cast<double>(__uint_as_float(x.y & 0xffff0000u));
+    for (int q = 0; q < OB / 128; ++q) {
+        const int64_t at = row * OB + 128 * q + 4 * lane;
+        const uint2 h = LQ_AT(reinterpret_cast<const uint2*>(ES + at)), m = LQ_AT(reinterpret_cast<const uint2*>(ES + r * OB + at)),
+                    l = LQ_AT(reinterpret_cast<const uint2*>(ES + 2 * r * OB + at));
+        const uint32_t hh[2] = {h.x, h.y}, mm[2] = {m.x, m.y}, ll[2] = {l.x, l.y};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {                   // the two lower terms add exactly, and the sum is the fp32 number they came from
+            const auto part = [&](const uint32_t (&x)[2]) { return __uint_as_float(u & 1 ? x[u / 2] & 0xffff0000u : x[u / 2] << 16); };
+            v[q][u] = part(hh) + (part(mm) + part(ll));
+            mx = fmaxf(mx, digit_mag(v[q][u]));
+        }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) mx = fmax(mx, digit_mag(v[u]));
-    mx = cta_max256(mx, red);
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const int e = isfinite(mx) ? exp_for8(mx) : 0;
-    if (threadIdx.x == 0) LQ_AT(scale + row) = isfinite(mx) ? ldexpf(1.0f, e) : __int_as_float(0x7fc00000);
-    store_digits<NS>(v, e, SL + row * OB + t, slice_bytes);
+    if (lane == 0) LQ_AT(scale + row) = isfinite(mx) ? ldexpf(1.0f, e) : __int_as_float(0x7fc00000);
+#pragma unroll
+    for (int q = 0; q < OB / 128; ++q) store_digits<NS>(v[q], e, SL + row * OB + 128 * q + 4 * lane, slice_bytes);
 }
 
 struct QuantOut {
@@ -559,7 +564,7 @@ int far_update(lq_handle* h, cudaStream_t st, const WsLayout& L, char* wsp, cons
     uint8_t* ED = reinterpret_cast<uint8_t*>(wsp + L.ed);
     float* cscale = reinterpret_cast<float*>(wsp + L.cscale);
     float* rscale = reinterpret_cast<float*>(wsp + L.rscale);
-    slice_errors_kernel<NS><<<static_cast<unsigned>(r), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(wsp + L.es), r, rscale, ED, r * OB);
+    slice_errors_kernel<NS><<<static_cast<unsigned>(lq_ceil_div(r, 8)), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(wsp + L.es), r, rscale, ED, r * OB);
     LQ_LAUNCH_CHECK();
     slice_cols_wide_kernel<NS><<<static_cast<unsigned>(lq_ceil_div(c - end, 32)), SC_THREADS, 0, st>>>(
         U + o0 * ldu, ldu, static_cast<int>(OB), end, c, nullptr, nullptr, cscale, UD, c * OB);
