@@ -395,6 +395,280 @@ inblock_kernel(const float* __restrict__ Wc, int64_t ldc, int64_t r, int64_t c, 
     }
 }
 
+// ------------------------------------------------------- the column loop, one thread per row ----
+// The same loop with a row in one thread: the block's 128 columns go in eight groups of 16.  A group's weights sit in
+// registers while its columns are quantised one after the other (their errors feed the rest of the group at once); the
+// groups behind wait in shared memory, transposed, and take a group's 16 errors in one pass through registers.  Only the
+// triangle is computed, a weight's nearest grid point is a bisection over registers, and nothing crosses lanes: a column
+// costs ~150 instructions per 32 rows where the warp-per-row kernel takes 450 and waits for a vote and two shuffles.  Every
+// weight receives the same fused multiply-adds in the same order, so codes and errors are the same to the bit.  (Groups of 32
+// take the same time with twice the code; four warps that share the work of 32 rows through shared memory and barriers took
+// 35 us at 28 rows per SM.)  ncu at 360 rows per SM: issue slots 38 %, shared memory 42 % (U comes as one broadcast read
+// per four columns), waits on those reads lead.
+constexpr int IR_GROUP = 16;
+constexpr int IR_MAX_ROWS = 368;             // rows per CTA that the shared memory holds
+constexpr int IR_MAX_THREADS = 384;          // 168 registers each
+
+struct RowArgs {
+    const float* Wc; int64_t ldc, r, c, i0;
+    const float* U; int64_t ldu;
+    const float* grid; const float* scale; const int32_t* zero; int group, n_groups;
+    int rows;                                // rows per CTA
+};
+
+template <int K, bool AFFINE>
+__global__ void __launch_bounds__(IR_MAX_THREADS, 1)
+inblock_rows_kernel(RowArgs A, QuantOut out) {
+    extern __shared__ float Us[];                          // B x B block of U, rows scaled by 1 / U_jj; then B reciprocals
+    float* invd = Us + B * B;
+    const int rows = A.rows;
+    float* Wt = invd + B;                                  // the columns behind the first group: Wt[(col - IR_GROUP) * rows + row]
+    const int tid = threadIdx.x, nthr = blockDim.x, lr = tid;              // lr: row within the CTA
+    const int64_t row = static_cast<int64_t>(blockIdx.x) * rows + lr;
+    const bool valid = lr < rows && row < A.r;
+    const int bw = (A.c - A.i0) < B ? static_cast<int>(A.c - A.i0) : B;
+
+    const bool whole = bw == B && (A.ldu % 4 == 0);
+    for (int idx = tid; idx < B * B / 4; idx += nthr) {
+        const int jj = idx / (B / 4), k4 = (idx % (B / 4)) * 4;
+        if (whole) {
+            const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(Us + jj * B + k4));
+            if (LQ_DBG_OK(A.U + (A.i0 + jj) * A.ldu + A.i0 + k4, 16) && LQ_DBG_OK(Us + jj * B + k4, 16))
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(A.U + (A.i0 + jj) * A.ldu + A.i0 + k4) : "memory");
+        } else {
+            float t[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int kk = k4 + u;
+                t[u] = (jj < bw && kk < bw) ? LQ_AT(A.U + (A.i0 + jj) * A.ldu + A.i0 + kk) : (jj == kk ? 1.0f : 0.0f);
+            }
+            LQ_AT(reinterpret_cast<float4*>(Us + jj * B + k4)) = make_float4(t[0], t[1], t[2], t[3]);
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+
+    // the row's weights: the first group into registers, the others transposed into shared memory; the working copy's rows
+    // start on 16-byte boundaries
+    float w[IR_GROUP];
+    auto fetch = [&](int g) {
+#pragma unroll
+        for (int k = 0; k < IR_GROUP; k += 4) {
+            const float* p = A.Wc + row * A.ldc + A.i0 + g * IR_GROUP + k;
+            const int col = g * IR_GROUP + k;
+            if (valid && col + 3 < bw) {
+                const float4 v = LQ_AT(reinterpret_cast<const float4*>(p));
+                w[k] = v.x; w[k + 1] = v.y; w[k + 2] = v.z; w[k + 3] = v.w;
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) w[k + u] = (valid && col + u < bw) ? LQ_AT(p + u) : 0.0f;
+            }
+        }
+    };
+    auto park = [&](int g) {
+#pragma unroll
+        for (int k = 0; k < IR_GROUP; ++k) Wt[((g - 1) * IR_GROUP + k) * rows + lr] = w[k];
+    };
+    if (lr < rows) {                       // four groups' loads in flight at a time
+#pragma unroll 1
+        for (int g0 = B / IR_GROUP - 4; g0 >= 0; g0 -= 4) {
+            float x[3][IR_GROUP];
+#pragma unroll
+            for (int q = 3; q > 0; --q) {
+                fetch(g0 + q);
+#pragma unroll
+                for (int k = 0; k < IR_GROUP; ++k) x[q - 1][k] = w[k];
+            }
+            fetch(g0);
+#pragma unroll
+            for (int q = 1; q < 4; ++q)
+#pragma unroll
+                for (int k = 0; k < IR_GROUP; ++k) Wt[((g0 + q - 1) * IR_GROUP + k) * rows + lr] = x[q - 1][k];
+            if (g0 > 0) park(g0);
+        }
+    }
+    // grid points and the midpoints between them, those in ascending order: the code is the number of midpoints below the weight
+    float gp[AFFINE ? 1 : K], mid[AFFINE ? 1 : K - 1];
+    float S = 1.0f, Z = 0.0f, rS = 1.0f;
+    if (!AFFINE) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) gp[k] = valid ? LQ_AT(A.grid + row * K + k) : 0.0f;
+        bool ascending = true;
+#pragma unroll
+        for (int k = 0; k < K - 1; ++k) mid[k] = 0.5f * (gp[k] + gp[k + 1]);
+#pragma unroll
+        for (int k = 0; k + 1 < K - 1; ++k) ascending = ascending && mid[k] <= mid[k + 1];
+        if (K > 2 && !ascending) {                         // a caller's own table: no weight lies above a NaN
+#pragma unroll
+            for (int k = 0; k < K - 1; ++k) mid[k] = mid[k] == mid[k] ? mid[k] : INFINITY;
+            for (int pass = 0; pass < K - 2; ++pass) {
+#pragma unroll
+                for (int k = 0; k + 1 < K - 1; ++k) {
+                    const float lo = fminf(mid[k], mid[k + 1]), hi = fmaxf(mid[k], mid[k + 1]);
+                    mid[k] = lo; mid[k + 1] = hi;
+                }
+            }
+        }
+    }
+    auto affine_params = [&](int col) {                    // of the group that column `col` of the block lies in
+        if (!valid || col >= bw) return;
+        const int64_t gi = (A.i0 + col) / A.group;
+        const int64_t gidx = row * A.n_groups + (gi < A.n_groups ? gi : A.n_groups - 1);
+        S = LQ_AT(A.scale + gidx);
+        Z = static_cast<float>(LQ_AT(A.zero + gidx));
+        rS = __fdiv_rn(1.0f, S);
+    };
+    const bool small_groups = AFFINE && A.group % IR_GROUP != 0;
+
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (nthr >= B) {
+        if (tid < B) LQ_AT(invd + tid) = 1.0f / LQ_AT(Us + tid * B + tid);
+    } else {
+        for (int j = tid; j < B; j += nthr) LQ_AT(invd + j) = 1.0f / LQ_AT(Us + j * B + j);
+    }
+    __syncthreads();
+    for (int idx = tid; idx < B * B / 4; idx += nthr) {
+        float4* p4 = reinterpret_cast<float4*>(Us) + idx;
+        float4 v = LQ_AT(p4);
+        const float sc = LQ_AT(invd + idx / (B / 4));
+        v.x *= sc; v.y *= sc; v.z *= sc; v.w *= sc;
+        LQ_AT(p4) = v;
+    }
+    __syncthreads();
+
+    // w[k] (column k of group g) takes the errors of group s
+    auto feed = [&](int s, int g, auto err) {
+#pragma unroll
+        for (int j = 0; j < IR_GROUP; ++j) {
+            const float d = err(j);
+            const float4* u4 = reinterpret_cast<const float4*>(Us + (s * IR_GROUP + j) * B + g * IR_GROUP);
+#pragma unroll
+            for (int k = 0; k < IR_GROUP; k += 4) {
+                const float4 u = u4[k / 4];
+                w[k] = fmaf(-d, u.x, w[k]);
+                w[k + 1] = fmaf(-d, u.y, w[k + 1]);
+                w[k + 2] = fmaf(-d, u.z, w[k + 2]);
+                w[k + 3] = fmaf(-d, u.w, w[k + 3]);
+            }
+        }
+    };
+    // E of group s as three bf16 terms, and the row's share of the loss
+    float loss = 0.0f;
+    auto emit = [&](int s, auto err) {
+        if (!valid) return;
+#pragma unroll
+        for (int k8 = 0; k8 < IR_GROUP; k8 += 8) {
+            uint32_t h[4], m[4], l[4];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) {
+                const int col = s * IR_GROUP + k8 + e;
+                const float e0 = col < bw ? err(k8 + e) * invd[col] : 0.0f, e1 = col + 1 < bw ? err(k8 + e + 1) * invd[col + 1] : 0.0f;
+                loss = fmaf(e0, e0, loss);
+                loss = fmaf(e1, e1, loss);
+                __nv_bfloat16 h0, m0, l0, h1, m1, l1;
+                lq_split3(e0, h0, m0, l0);
+                lq_split3(e1, h1, m1, l1);
+                h[e / 2] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+                m[e / 2] = static_cast<uint32_t>(__bfloat16_as_ushort(m0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(m1)) << 16);
+                l[e / 2] = static_cast<uint32_t>(__bfloat16_as_ushort(l0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
+            }
+            __nv_bfloat16* p = out.esplit + row * out.e_ld + out.e_col + s * IR_GROUP + k8;
+            LQ_AT(reinterpret_cast<uint4*>(p)) = make_uint4(h[0], h[1], h[2], h[3]);
+            LQ_AT(reinterpret_cast<uint4*>(p + A.r * out.e_ld)) = make_uint4(m[0], m[1], m[2], m[3]);
+            LQ_AT(reinterpret_cast<uint4*>(p + 2 * A.r * out.e_ld)) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+    };
+
+#pragma unroll 1
+        for (int s = 0; s < B / IR_GROUP; ++s) {
+            uint32_t codes[IR_GROUP / 4];
+            if (AFFINE && !small_groups) affine_params(s * IR_GROUP);
+            // quantise the group's columns in order; w[j] becomes the error w - q
+#pragma unroll
+            for (int j = 0; j < IR_GROUP; ++j) {
+                if (AFFINE && j % 4 == 0 && small_groups) affine_params(s * IR_GROUP + j);
+                int code;
+                float qv, d;
+                if (AFFINE) {
+                    float qi = rintf(w[j] * rS) + Z;
+                    qi = fminf(fmaxf(qi, 0.0f), static_cast<float>(K - 1));
+                    code = static_cast<int>(qi);
+                    qv = (qi - Z) * S;
+                    d = fmaf(-(qi - Z), S, w[j]);
+                } else {
+                    float mm[AFFINE ? 1 : K - 1], gg[AFFINE ? 1 : K];
+#pragma unroll
+                    for (int k = 0; k < K - 1; ++k) mm[k] = mid[k];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) gg[k] = gp[k];
+                    code = 0;
+#pragma unroll
+                    for (int n = K / 2; n >= 1; n /= 2) {
+                        const bool up = w[j] > mm[n - 1];
+                        code = 2 * code + (up ? 1 : 0);
+#pragma unroll
+                        for (int k = 0; k < n; ++k) {
+                            if (k < n - 1) mm[k] = up ? mm[n + k] : mm[k];
+                            gg[k] = up ? gg[n + k] : gg[k];
+                        }
+                    }
+                    qv = gg[0];
+                    d = w[j] - qv;
+                }
+                if (j % 4 == 0) codes[j / 4] = static_cast<uint32_t>(code);
+                else codes[j / 4] |= static_cast<uint32_t>(code) << (8 * (j % 4));
+                if (out.what && valid && s * IR_GROUP + j < bw) {
+                    const int64_t at = row * out.ldwh + A.i0 + s * IR_GROUP + j;
+                    if (out.what_bf16) LQ_AT(static_cast<__nv_bfloat16*>(out.what) + at) = __float2bfloat16_rn(qv);
+                    else LQ_AT(static_cast<float*>(out.what) + at) = qv;
+                }
+                w[j] = d;
+                const float* u = Us + (s * IR_GROUP + j) * B + s * IR_GROUP;
+#pragma unroll
+                for (int k = (j + 1) & ~3; k < IR_GROUP; k += 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(u + k);
+                    if (k > j) w[k] = fmaf(-d, x.x, w[k]);
+                    if (k + 1 > j) w[k + 1] = fmaf(-d, x.y, w[k + 1]);
+                    if (k + 2 > j) w[k + 2] = fmaf(-d, x.z, w[k + 2]);
+                    if (k + 3 > j) w[k + 3] = fmaf(-d, x.w, w[k + 3]);
+                }
+            }
+            if (valid) {
+                uint8_t* cp = out.codes + row * A.c + A.i0 + s * IR_GROUP;
+                if (A.c % 16 == 0 && (s + 1) * IR_GROUP <= bw) {
+                    LQ_AT(reinterpret_cast<uint4*>(cp)) = make_uint4(codes[0], codes[1], codes[2], codes[3]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < IR_GROUP; k += 4) {
+                        const int col = s * IR_GROUP + k;
+                        if (A.c % 4 == 0 && col + 3 < bw) LQ_AT(reinterpret_cast<uint32_t*>(cp + k)) = codes[k / 4];
+                        else {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (col + u < bw) LQ_AT(cp + k + u) = static_cast<uint8_t>((codes[k / 4] >> (8 * u)) & 0xff);
+                        }
+                    }
+                }
+            }
+            {
+                float d[IR_GROUP];
+#pragma unroll
+                for (int k = 0; k < IR_GROUP; ++k) d[k] = w[k];
+                emit(s, [&](int k) { return d[k]; });
+                if (lr < rows) {
+#pragma unroll 1
+                    for (int g = B / IR_GROUP - 1; g > s; --g) {           // the next group last: it stays in registers
+#pragma unroll
+                        for (int k = 0; k < IR_GROUP; ++k) w[k] = Wt[((g - 1) * IR_GROUP + k) * rows + lr];
+                        feed(s, g, [&](int j) { return d[j]; });
+                        if (g > s + 1) park(g);
+                    }
+                }
+            }
+        }
+        if (valid) LQ_AT(out.loss_rows + row) += static_cast<double>(loss);
+}
+
 // Packed output: the b-bit codes of a row as one little-endian bit stream (code j in bits
 // [j b, (j + 1) b) of the row), one thread per output byte.
 __global__ void pack_codes_kernel(const uint8_t* __restrict__ codes, int64_t r, int64_t c, int bits,
@@ -516,12 +790,36 @@ int launch_inblock_rows(cudaStream_t st, int sm_count, float* Wc, int64_t ldc, i
     LQ_LAUNCH_CHECK();
     return LQ_OK;
 }
+// The thread-per-row kernel: one CTA per SM with an even share of the rows.  A launch takes ~30 us however few the rows (one
+// warp's chain), where the warp-per-row kernel takes 18 at 28 rows per SM, 27 at 55, 50 at 97 and 149 at 360; this one takes 30
+// at 97 and 74 at 360: the line is at 60 rows per SM.
+template <int K, bool AFFINE>
+int launch_inblock_by_rows(cudaStream_t st, int sm_count, const RowArgs& args, const QuantOut& out) {
+    RowArgs a = args;
+    constexpr int base = (B * B + B) * static_cast<int>(sizeof(float));
+    static lq_once_per_device attr_set;
+    if (attr_set.first()) {
+        LQ_CUDA_TRY(cudaFuncSetAttribute(inblock_rows_kernel<K, AFFINE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         base + (B - IR_GROUP) * IR_MAX_ROWS * static_cast<int>(sizeof(float))));
+    }
+    const int64_t rounds = lq_ceil_div(a.r, static_cast<int64_t>(sm_count) * IR_MAX_ROWS);
+    a.rows = static_cast<int>(lq_ceil_div(a.r, rounds * sm_count));
+    const unsigned threads = static_cast<unsigned>(lq_ceil_div(a.rows, 32) * 32);
+    const int smem = base + (B - IR_GROUP) * a.rows * static_cast<int>(sizeof(float));
+    inblock_rows_kernel<K, AFFINE><<<static_cast<unsigned>(lq_ceil_div(a.r, a.rows)), threads, smem, st>>>(a, out);
+    LQ_LAUNCH_CHECK();
+    return LQ_OK;
+}
 // A warp carries two rows where an SM gets enough of them to stay busy that way (measured: 2 % faster at 28 rows per
 // SM, 6 % at 360, 5 % slower at 14), and one where it refits groups inside the kernel.
 template <int K, bool AFFINE, bool REFIT>
 int launch_inblock(cudaStream_t st, int sm_count, float* Wc, int64_t ldc, int64_t r, int64_t c, int64_t i0, const float* U, int64_t ldu,
                    const float* grid, const float* scale, const int32_t* zero, int group, int n_groups, const QuantOut& out,
                    const RefitArgs& refit) {
+    if (!REFIT && r > 60 * static_cast<int64_t>(sm_count)) {
+        const RowArgs a = {Wc, ldc, r, c, i0, U, ldu, grid, scale, zero, group, n_groups, 0};
+        return launch_inblock_by_rows<K, AFFINE>(st, sm_count, a, out);
+    }
     if (!REFIT && r >= 24 * static_cast<int64_t>(sm_count))
         return launch_inblock_rows<K, AFFINE, REFIT, REFIT ? 1 : IB_ROWS>(st, sm_count, Wc, ldc, r, c, i0, U, ldu, grid, scale, zero, group, n_groups, out, refit);
     return launch_inblock_rows<K, AFFINE, REFIT, 1>(st, sm_count, Wc, ldc, r, c, i0, U, ldu, grid, scale, zero, group, n_groups, out, refit);

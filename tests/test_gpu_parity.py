@@ -492,6 +492,38 @@ def test_stage4_affine_isolated(lq, h, r, c, bits, group):
     assert abs(loss / loss_o - 1) <= LOSS_TOL
 
 
+@pytest.mark.parametrize("c,bits,group,copies", [(72, 4, 0, 1473), (200, 3, 0, 251), (1160, 2, 0, 251), (2100, 4, 0, 251), (1160, 4, 8, 251),
+                                                 (256, 2, 256, 251), (384, 3, 96, 400)])
+def test_stage4_tall_layers_row_for_row(lq, h, c, bits, group, copies):
+    """From 60 rows per SM on a row of the column loop belongs to one thread instead of one warp: the same arithmetic in the
+    same order, so a tall layer made of copies of a short one has the short one's codes and weights to the bit (one and two
+    rounds of CTAs, ragged last blocks, groups that start inside a group of 16 columns, a table that does not ascend)."""
+    g = torch.Generator().manual_seed(c + bits)
+    n0, K = 37, 1 << bits
+    W = torch.randn(n0, c, generator=g) * 0.02
+    U32 = torch.triu(torch.randn(c, c, generator=g)) * 0.05 + torch.diag(0.5 + torch.rand(c, generator=g))
+    cfg = lq.Config.make(grid="affine" if group else "nonuniform", bits=bits, group=group, T=40, t=8)
+    out = []
+    if group:
+        grid, scale = None, torch.rand(n0, c // group, generator=g) * 0.004 + 0.003
+        zero = torch.randint(0, K, (n0, c // group), generator=g, dtype=torch.int32)
+    else:
+        grid, scale, zero = torch.randn(n0, K, generator=g) * 0.03, None, None
+        if c != 200:
+            grid = torch.sort(grid, dim=1).values
+    for k in (1, copies):
+        t = lambda x: None if x is None else x.repeat(k, 1).cuda()
+        codes = torch.empty(n0 * k, c, dtype=torch.uint8, device="cuda")
+        what = torch.empty(n0 * k, c, device="cuda")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        ws = ws_for(lq, lq.lq_quantize_layer_workspace(cfg, n0 * k, c))
+        lq.lq_quantize_layer(h, cfg, t(W), U32.cuda(), codes, ws, t(grid), t(scale), t(zero), what, loss)
+        lq.lq_sync_status(h)
+        out.append((codes.view(k, n0, c), what.view(k, n0, c), loss.item() / k))
+    assert torch.equal(out[1][0], out[0][0].expand(copies, -1, -1)) and torch.equal(out[1][1], out[0][1].expand(copies, -1, -1))
+    np.testing.assert_allclose(out[1][2], out[0][2], rtol=1e-6)          # per block a row's fp32 sum of squares in another order
+
+
 @pytest.mark.parametrize("grid_type", ["nonuniform", "affine"])
 def test_stage4_many_rows_odd_count(lq, h, grid_type):
     """From 24 rows per SM on a warp of the in-block kernel carries two rows: an odd row count (the last warp has one
