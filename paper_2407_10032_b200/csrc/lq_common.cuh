@@ -204,6 +204,9 @@ struct lq_tc_gemm_args {
     // read up to the end of the last tile: N rounded up to 256 entries)
     const float* row_scale;
     const float* col_scale;
+    // bf16 operands stored the other way round: A_all / B_all hold rows of k (a_rows / b_rows of them, M / N entries each; rows beyond
+    // them read as zero); one pass
+    int mn_major;
     int spare_sms;   // SMs that the launch leaves to kernels on other streams (a persistent CTA keeps its SM until the launch ends)
 };
 int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a);

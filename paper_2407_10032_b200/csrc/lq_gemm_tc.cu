@@ -55,6 +55,8 @@ template <int CTAS> struct Cfg {
     static constexpr int TILE_M = BM * CTAS;
     // Instruction descriptor: D fp32, A and B bf16, both K-major, M = TILE_M, N = 256.
     static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(TILE_M >> 4) << 24);
+    // Both operands MN-major (rows of k): bits 15 and 16.
+    static constexpr uint32_t IDESC_MN = IDESC | (1u << 15) | (1u << 16);
     // The same for kind::i8: D int32 (2 in bits 4-5), A and B unsigned (0) or signed (1) 8-bit integers in bits 7-9 / 10-12.
     static constexpr uint32_t idesc_i8(bool a_signed, bool b_signed) {
         return (2u << 4) | ((a_signed ? 1u : 0u) << 7) | ((b_signed ? 1u : 0u) << 10) | (uint32_t(BN >> 3) << 17) |
@@ -286,6 +288,19 @@ __device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same for an MN-major bf16 tile: boxes of 64 entries of M (or N) by 64 rows of k, each a stack of 128-byte rows (8192 bytes);
+// groups of 8 rows of k are 1024 bytes apart, the next 64 entries of M one box further.
+constexpr int MN_BOX = 64, MN_BOX_BYTES = MN_BOX * BK * 2;
+__device__ __forceinline__ uint64_t make_desc_sw128_mn(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
+    d |= static_cast<uint64_t>(MN_BOX_BYTES >> 4) << 16;        // leading byte offset: to the next 64 entries of M
+    d |= static_cast<uint64_t>(1024 >> 4) << 32;                // stride byte offset: to the next 8 rows of k
+    d |= static_cast<uint64_t>(1) << 46;
+    d |= static_cast<uint64_t>(2) << 61;
+    return d;
+}
+
 // Map the idx-th scheduled tile to (tile row, tile column).  With upper_only, row tm keeps
 // the columns tn with (tn + 1) * BN > tm * tile_m.  The tiles are ordered in bands of `band`
 // tile rows, column by column inside a band: the CTAs of one scheduling round then work on a
@@ -378,10 +393,10 @@ __device__ __forceinline__ void seg_item(const Seg& g, int q, int& pass, int& kb
     kb = g.kb0 + kit - ps * g.kbn;
 }
 
-// MODE: BF16 operands, 8-bit integer operands whose sums go out by themselves (INT8_SUMS: stage 2), or 8-bit integer operands
+// MODE: BF16 operands (BF16_MN: stored as rows of k), 8-bit integer operands whose sums go out by themselves (INT8_SUMS: stage 2), or 8-bit integer operands
 // whose sum is scaled by row and column and added to D (INT8_SCALED: stage 4).  Each carries its own code only: the epilogue
 // holds 128 running sums per thread and spills with every register more (4 % of a launch for the bf16 form).
-enum { BF16 = 0, INT8_SUMS = 1, INT8_SCALED = 2 };
+enum { BF16 = 0, INT8_SUMS = 1, INT8_SCALED = 2, BF16_MN = 3 };
 template <int CTAS, int MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
@@ -390,7 +405,7 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     typedef Cfg<CTAS> C;
     constexpr int STAGES = C::STAGES;
     constexpr bool PAIR = CTAS == 2;
-    constexpr bool I8 = MODE != BF16, SUMS = MODE == INT8_SUMS, SCALED = MODE == INT8_SCALED;
+    constexpr bool MN = MODE == BF16_MN, I8 = MODE != BF16 && !MN, SUMS = MODE == INT8_SUMS, SCALED = MODE == INT8_SCALED;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[3 * MAX_STAGES + 4];
     __shared__ uint32_t tmem_base_slot;
@@ -461,7 +476,21 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     const int k0 = kb * p.bk_elems;
                     const uint32_t sa = smem_base + stage * C::STAGE_BYTES;
                     const uint32_t sb = sa + A_STAGE_BYTES;
-                    if (!PAIR) {
+                    if (MN) {
+                        uint32_t bar = bar_full + 8 * stage;
+                        if (mma_cta) mbar_arrive_expect_tx(bar, CTAS * C::STAGE_BYTES + p.stall_bytes);
+                        if (PAIR) bar = cluster_addr(bar, 0);
+#pragma unroll
+                        for (int b = 0; b < BM / MN_BOX; ++b) {
+                            if (PAIR) tma_load_2d_pair(sa + b * MN_BOX_BYTES, &map_a, bar, m0 + b * MN_BOX, k0);
+                            else tma_load_2d(sa + b * MN_BOX_BYTES, &map_a, bar, m0 + b * MN_BOX, k0);
+                        }
+#pragma unroll
+                        for (int b = 0; b < C::B_ROWS / MN_BOX; ++b) {
+                            if (PAIR) tma_load_2d_pair(sb + b * MN_BOX_BYTES, &map_b, bar, n0 + b * MN_BOX, k0);
+                            else tma_load_2d(sb + b * MN_BOX_BYTES, &map_b, bar, n0 + b * MN_BOX, k0);
+                        }
+                    } else if (!PAIR) {
                         mbar_arrive_expect_tx(bar_full + 8 * stage, C::STAGE_BYTES + p.stall_bytes);
                         tma_load_2d(sa, &map_a, bar_full + 8 * stage, k0, p.a_off[pass] + m0);
                         tma_load_2d(sb, &map_b, bar_full + 8 * stage, k0, p.b_off[pass] + n0);
@@ -505,10 +534,13 @@ lq_tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     tc_fence_after();
                     if (lane == 0) {
                         const uint32_t sa = smem_base + stage * C::STAGE_BYTES;
-                        const uint64_t da = make_desc_sw128(sa);
-                        const uint64_t db = make_desc_sw128(sa + A_STAGE_BYTES);
+                        const uint64_t da = MN ? make_desc_sw128_mn(sa) : make_desc_sw128(sa);
+                        const uint64_t db = MN ? make_desc_sw128_mn(sa + A_STAGE_BYTES) : make_desc_sw128(sa + A_STAGE_BYTES);
+                        if (MN) {
 #pragma unroll
-                        if (I8) {
+                            for (int kk = 0; kk < BK / UMMA_K; ++kk)      // 16 rows of k = 2048 bytes further
+                                umma_bf16<CTAS>(tmem_d, da + 128 * kk, db + 128 * kk, C::IDESC_MN, (q > 0 || kk > 0) ? 1u : 0u);
+                        } else if (I8) {
                             int pass, kb;
                             seg_item(seg, q, pass, kb);
                             const uint32_t idesc = p.idesc_pass[pass];
@@ -710,7 +742,8 @@ int max_pairs(int sm_count) {
     cached = 0;
     if (cudaFuncSetAttribute(lq_tc_gemm_kernel<2, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(lq_tc_gemm_kernel<2, INT8_SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, INT8_SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess) {
+        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, INT8_SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(lq_tc_gemm_kernel<2, BF16_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return cached;
     }
@@ -751,6 +784,7 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
         LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, INT8_SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
         LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, INT8_SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
+        LQ_CUDA_TRY(cudaFuncSetAttribute(lq_tc_gemm_kernel<1, BF16_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES));
     }
     // The pair form pays off once there are at least a few 256-row tiles; below that one CTA per tile.
     const int pairs = (a.M > BM) ? max_pairs(h->sm_count) : 0;
@@ -767,8 +801,12 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
     const int bk_elems = i8 ? 2 * BK : BK;                 // a k-step is one 128-byte swizzle row of either type
     const CUtensorMapDataType op_dt = i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const int op_bytes = i8 ? 1 : 2;
-    if (!make_map_2d(&map_a, op_dt, op_bytes, a.A_all, a.K, a.a_rows, a.lda, bk_elems, BM) ||
-        !make_map_2d(&map_b, op_dt, op_bytes, a.B_all, a.K, a.b_rows, a.ldb, bk_elems, b_rows_box) ||
+    if (a.mn_major && (i8 || a.hole || a.n_lvl || a.n_pass > 1)) return LQ_ERR_INVALID_ARG;
+    const bool maps = a.mn_major ? make_map_2d(&map_a, op_dt, op_bytes, a.A_all, a.M, a.a_rows, a.lda, MN_BOX, BK) &&
+                                       make_map_2d(&map_b, op_dt, op_bytes, a.B_all, a.N, a.b_rows, a.ldb, MN_BOX, BK)
+                                 : make_map_2d(&map_a, op_dt, op_bytes, a.A_all, a.K, a.a_rows, a.lda, bk_elems, BM) &&
+                                       make_map_2d(&map_b, op_dt, op_bytes, a.B_all, a.K, a.b_rows, a.ldb, bk_elems, b_rows_box);
+    if (!maps ||
         !make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.D, n_all, a.M, a.ldd, EPI_COLS, BM))
         return LQ_ERR_CUDA;
     map_d1 = map_d2 = map_d;
@@ -875,7 +913,7 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        const auto kernel = !i8 ? lq_tc_gemm_kernel<2, BF16> : a.row_scale ? lq_tc_gemm_kernel<2, INT8_SCALED> : lq_tc_gemm_kernel<2, INT8_SUMS>;
+        const auto kernel = a.mn_major ? lq_tc_gemm_kernel<2, BF16_MN> : !i8 ? lq_tc_gemm_kernel<2, BF16> : a.row_scale ? lq_tc_gemm_kernel<2, INT8_SCALED> : lq_tc_gemm_kernel<2, INT8_SUMS>;
         const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, map_d, map_d1, map_d2, p);
         if (le != cudaSuccess) {
             cudaGetLastError();
@@ -883,7 +921,7 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
         }
         lq_launches_total.fetch_add(1, std::memory_order_relaxed);
     } else {
-        const auto kernel = !i8 ? lq_tc_gemm_kernel<1, BF16> : a.row_scale ? lq_tc_gemm_kernel<1, INT8_SCALED> : lq_tc_gemm_kernel<1, INT8_SUMS>;
+        const auto kernel = a.mn_major ? lq_tc_gemm_kernel<1, BF16_MN> : !i8 ? lq_tc_gemm_kernel<1, BF16> : a.row_scale ? lq_tc_gemm_kernel<1, INT8_SCALED> : lq_tc_gemm_kernel<1, INT8_SUMS>;
         kernel<<<active, NUM_THREADS, Cfg<1>::SMEM_BYTES, stream>>>(map_a, map_b, map_d, map_d1, map_d2, p);
         LQ_LAUNCH_CHECK();
     }

@@ -150,6 +150,23 @@ def test_stage1_token_major(lq, h, c, n, dtype):
     assert np.max(np.abs(Hg - Href) / scale) < 5e-6
 
 
+@pytest.mark.parametrize("c,n,pad,dtype", [(64, 64, 0, torch.bfloat16), (300, 63, 4, torch.bfloat16), (1032, 520, 0, torch.bfloat16),
+                                           (260, 129, 12, torch.bfloat16), (520, 64, 3, torch.float32)])
+def test_stage1_token_rows_where_they_stand(lq, h, c, n, pad, dtype):
+    """Rows of tokens contracted without a transpose (MN-major operands, boxes of 64 features by 64 tokens): features and
+    tokens at the edges of boxes, tiles and k-steps, strided rows."""
+    g = torch.Generator().manual_seed(c + n)
+    Xt = torch.randn(n, c + pad, generator=g).to(dtype).cuda()[:, :c]
+    H = torch.zeros(c, c, device="cuda")
+    ws = ws_for(lq, lq.lq_hessian_workspace(dtype, c, n, token_major=True))
+    lq.lq_hessian_accumulate(h, Xt, H, 2.0, ws, token_major=True)
+    lq.lq_hessian_finalize(h, H)
+    lq.lq_sync_status(h)
+    Href = O.hessian(f64(Xt).T.copy())
+    scale = np.sqrt(np.outer(np.diag(Href), np.diag(Href)))
+    assert np.max(np.abs(f64(H) - Href) / scale) < 5e-6
+
+
 def test_stage1_chunks_add_up(lq, h):
     g = torch.Generator().manual_seed(5)
     X = torch.randn(256, 4096, generator=g).bfloat16().cuda()
