@@ -697,12 +697,18 @@ kmeans_rows_kernel(const T* __restrict__ W, int64_t ldw, int64_t r, int64_t c, c
                 for (int k = 0; k < K; ++k) { red[warp][k] = ns[k]; red[warp][K + k] = nsw[k]; }
             }
             __syncthreads();
+            bool moved = false;
             if (tid < K) {
                 double den = 0.0, num = 0.0;
                 for (int w = 0; w < KM_WARPS; ++w) { den += red[w][tid]; num += red[w][K + tid]; }
-                if (den > 0.0) g[tid] = num / den;      // an empty / weightless cluster keeps its centroid
+                if (den > 0.0) {                        // an empty / weightless cluster keeps its centroid
+                    const double v = num / den;
+                    moved = v != g[tid];
+                    g[tid] = v;
+                }
             }
-            __syncthreads();
+            // no centroid moved: every further iteration would form the same sums in the same order and the same centroids
+            if (!__syncthreads_or(moved)) break;
         }
         if (tid < K) LQ_AT(grid + row * K + tid) = static_cast<float>(g[tid]);
         __syncthreads();

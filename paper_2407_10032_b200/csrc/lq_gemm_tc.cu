@@ -894,7 +894,9 @@ int lq_tc_gemm(lq_handle* h, cudaStream_t stream, const lq_tc_gemm_args& a) {
     p.k_parts = 1;
     if (a.accumulate && p.segs_per_tile >= 16) {          // long K only: every unit pays one epilogue
         double best = static_cast<double>(lq_ceil_div(p.num_tiles, workers));
-        for (int q = 2; q <= 8 && q <= p.segs_per_tile; ++q) {
+        // more than 8 parts only where 8 do not give every worker a unit (512 features: 3 tiles, 24 parts)
+        const int most = 8 * p.num_tiles < workers ? workers / p.num_tiles : 8;
+        for (int q = 2; q <= most && q <= p.segs_per_tile; ++q) {
             const double t = static_cast<double>(lq_ceil_div(static_cast<int64_t>(p.num_tiles) * q, workers)) / q;
             if (t < best * 0.98) { best = t; p.k_parts = q; }
         }

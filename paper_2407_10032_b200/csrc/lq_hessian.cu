@@ -16,11 +16,30 @@ __global__ void split3_kernel(const float* __restrict__ src, int64_t ld, int64_t
     __nv_bfloat16* d0 = dst + row * dst_ld;
     __nv_bfloat16* d1 = d0 + rows * dst_ld;
     __nv_bfloat16* d2 = d1 + rows * dst_ld;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < dst_ld; j += (int64_t)gridDim.x * blockDim.x) {
-        float x = j < cols ? LQ_AT(s + j) : 0.0f;
-        __nv_bfloat16 a, b, c;
-        lq_split3(x, a, b, c);
-        LQ_AT(d0 + j) = a; LQ_AT(d1 + j) = b; LQ_AT(d2 + j) = c;
+    // eight entries per thread, 16-byte stores (dst_ld is a multiple of 8); 16-byte loads where the source rows allow them
+    const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+    for (int64_t j = 8 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); j < dst_ld; j += 8 * (int64_t)gridDim.x * blockDim.x) {
+        float x[8];
+        if (vec && j + 8 <= cols) {
+            const float4 u = LQ_AT(reinterpret_cast<const float4*>(s + j)), v = LQ_AT(reinterpret_cast<const float4*>(s + j) + 1);
+            x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = j + e < cols ? LQ_AT(s + j + e) : 0.0f;
+        }
+        uint32_t t[3][4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            __nv_bfloat16 a[2][3];
+            lq_split3(x[e], a[0][0], a[0][1], a[0][2]);
+            lq_split3(x[e + 1], a[1][0], a[1][1], a[1][2]);
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                t[q][e / 2] = static_cast<uint32_t>(__bfloat16_as_ushort(a[0][q])) | (static_cast<uint32_t>(__bfloat16_as_ushort(a[1][q])) << 16);
+        }
+        LQ_AT(reinterpret_cast<uint4*>(d0 + j)) = make_uint4(t[0][0], t[0][1], t[0][2], t[0][3]);
+        LQ_AT(reinterpret_cast<uint4*>(d1 + j)) = make_uint4(t[1][0], t[1][1], t[1][2], t[1][3]);
+        LQ_AT(reinterpret_cast<uint4*>(d2 + j)) = make_uint4(t[2][0], t[2][1], t[2][2], t[2][3]);
     }
 }
 
@@ -173,7 +192,7 @@ extern "C" int lq_hessian_accumulate(lq_handle* h, void* stream, const void* X, 
     } else {
         if (c > 65535) return LQ_ERR_UNSUPPORTED;        // rows of the split / transpose launches ride on the second grid dimension
         if (!token_major) {
-            dim3 grid(static_cast<unsigned>(lq_ceil_div(ld, 256) < 64 ? lq_ceil_div(ld, 256) : 64), static_cast<unsigned>(c));
+            dim3 grid(static_cast<unsigned>(lq_ceil_div(ld, 2048) < 64 ? lq_ceil_div(ld, 2048) : 64), static_cast<unsigned>(c));
             split3_kernel<<<grid, 256, 0, st>>>(static_cast<const float*>(X), ldx, c, n_chunk, staged, ld);
         } else {
             dim3 grid(static_cast<unsigned>(lq_ceil_div(ld, 32)), static_cast<unsigned>(lq_ceil_div(c, 32)));

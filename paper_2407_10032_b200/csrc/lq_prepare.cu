@@ -19,25 +19,23 @@
 // Every product has inner dimension 128 and all of a step's updates form one launch over the
 // whole width, so the grid stays large from the first step to the last.
 //
-// The matrix, the diagonal blocks and the panels are fp64 (fp32 factors of an ill-conditioned H move
-// too many quantisation decisions).  The updates are done in two levels over outer blocks of
-// OBB = 8 block columns (1024 columns):
-//   eager    : the rows and the columns of the current outer block get every step's update at once, on the
-//              FP64 tensor-core MMA (mma.sync m8n8k4 f64) fed by a cp.async ring -- these are the tiles the
-//              outer block's own diagonal and panel kernels read;
-//   deferred : all other tiles (rows above the outer block, columns outside it) get the updates of the outer
-//              block's steps in one product of inner dimension 1024 when the outer block is complete, on the
-//              integer tensor cores (tcgen05 kind::i8, lq_tc_gemm).  The fp64 operands are cut into S = 5 slices of
-//              balanced 8-bit integer digits below a per-row power of two; a product of two slices is a sum of
-//              integers that the int32 accumulator holds exactly, the leading slice pair (s = t = 1) is kept as a
-//              result of its own and the other pairs with s + t <= S + 1 are combined, least significant level first,
-//              in fp32; the two results are added in fp64 and scaled back (15 integer products in all).  Worth ~39 bits
-//              relative to the largest entry of a row; entries of one row of a panel differ by several bits, which is
-//              why four slices are not enough (U then comes out 1e-7 to 5e-7 of its largest entry off, measured here and
-//              in the CPU emulation alike; five hold it to 1e-8).  An fp32 accumulation of split floating-point
-//              operands keeps ~20 bits whatever the number of terms and moves 0.1 - 0.2 % of the codes.  The same
-//              slices as bf16 values on the bf16 path (exact in its fp32 accumulator per 128 of the inner dimension)
-//              remain selectable for tests; the integer path runs the stage 1.2 - 1.5 x faster.
+// The matrix and the diagonal blocks are fp64 (fp32 factors of an ill-conditioned H move too many quantisation decisions).
+// Matrices below 48 blocks (6144 columns) are bound by the serial chain of diagonal blocks and stay on the FP64 tensor-core
+// MMA (mma.sync m8n8k4 f64, fed by a cp.async ring) throughout.  Wider ones are swept in outer blocks of OBB = 8 block columns
+// (1024 columns): only an outer block's own 1024 x 1024 diagonal part goes through the steps above; its panels, the final rows
+// of U beside it and the updates of all other tiles are products of inner dimension 1024 on the integer tensor cores
+// (tcgen05 kind::i8, lq_tc_gemm), see wide_sweep().  The fp64 operands are cut into balanced 8-bit integer digits below a
+// per-row power of two; the digit products of one level sum exactly in int32.
+//   far tiles : 5 digits, 15 products; the leading pair (s = t = 1) is a result of its own, the levels s + t = 3 .. 6 are
+//               combined, least significant first, in fp32, and the two are added in fp64.  Worth ~39 bits relative to the
+//               largest entry of a row; entries of one row of a panel differ by several bits, which is why four slices are
+//               not enough (U then comes out 1e-7 to 5e-7 of its largest entry off, measured here and in the CPU emulation
+//               alike; five hold it to 1e-8).
+//   panels, rows of U : 6 digits, 21 products, two exact leading levels (they are products with the inverse factor V, whose
+//               entries are up to sqrt(cond) larger than the results').
+// An fp32 accumulation of split floating-point operands keeps ~20 bits whatever the number of terms and moves 0.1 - 0.2 % of the
+// codes.  The older form with the outer block's rows and columns updated step by step on the FP64 MMA and the far tiles' slices as
+// bf16 values remains selectable for tests.
 #include "lq_common.cuh"
 #include "lq_digits.cuh"
 
@@ -696,13 +694,20 @@ finalize_kernel(const double* __restrict__ A, int64_t cp, int64_t c, float* __re
     const int64_t i1 = i0 + FIN_ROWS < c ? i0 + FIN_ROWS : c;
     double s = 0.0;
     if (j < c) {
-        for (int64_t i = i0 + ty; i < i1; i += 8) {
-            double u = 0.0;
-            if (i <= j) {
-                u = LQ_AT(A + i * cp + j);
-                s = fma(u, u, s);
+        // eight rows' reads in flight (one at a time, a column of 32 rows was 32 trips to the L2: 18 us at c = 512)
+        for (int64_t ib = i0 + ty; ib < i1; ib += 64) {
+            double u[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t i = ib + 8 * e;
+                u[e] = (i < i1 && i <= j) ? LQ_AT(A + i * cp + j) : 0.0;
             }
-            LQ_AT(U + i * ldu + j) = static_cast<float>(u);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t i = ib + 8 * e;
+                s = fma(u[e], u[e], s);
+                if (i < i1) LQ_AT(U + i * ldu + j) = static_cast<float>(u[e]);
+            }
         }
     }
     red[ty][tx] = s;

@@ -64,13 +64,13 @@ __global__ void to_f32_kernel(const T* __restrict__ W, int64_t ldw, int64_t c, f
     }
 }
 
-// UT[s][n][k - o] = s-th bf16 term of U[k][n] for the rows k of column n's own outer block, which starts at o (three stacked
-// c x ldt matrices): the right operand of the products inside an outer block.  64 x 64 tiles: 16-byte reads along n, 16-byte
+// UT[s][n][k - o] = s-th bf16 term of U[k][n] (three stacked c x ldt matrices), the right operand of the bf16 products.  With
+// `band` for the rows k of column n's own outer block only, which starts at o; else for all k, o = 0.  64 x 64 tiles: 16-byte reads along n, 16-byte
 // writes (eight bf16) along k.
 __global__ void __launch_bounds__(256)
-split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv_bfloat16* __restrict__ UT, int64_t ldt) {
+split_transpose_kernel(const float* __restrict__ U, int64_t ldu, int64_t c, __nv_bfloat16* __restrict__ UT, int64_t ldt, int band) {
     __shared__ float tile[64][65];
-    const int64_t n0 = (int64_t)blockIdx.x * 64, o = n0 / OB * OB, k0 = o + (int64_t)blockIdx.y * 64;
+    const int64_t n0 = (int64_t)blockIdx.x * 64, o = band ? n0 / OB * OB : 0, k0 = o + (int64_t)blockIdx.y * 64;
     if (k0 > n0) return;                                // below the diagonal: zero, and never read
     const int tid = threadIdx.x;
     const bool vec_in = (ldu % 4 == 0) && ((reinterpret_cast<uintptr_t>(U) & 15) == 0);
@@ -739,18 +739,23 @@ constexpr int FAR_SLICES = 4;            // digits per operand of the products b
 struct WsLayout {
     size_t wc, ut, es, loss, ud, ed, cscale, rscale, total;
     int64_t ldc, ldt;
+    bool digits;             // products beyond an outer block as digits; the bf16 terms of U for its diagonal blocks only
 };
+// From this many weights on the products beyond an outer block go as digits: 4096 x 14336 and larger gain (and run at the power
+// limit), 4096 x 4096 is even (three such products, 98 us with their slicing against 89), 1000 x 1412 loses 15 of 1370 us.
+constexpr int64_t DIGITS_MIN_WEIGHTS = 24ll << 20;
 WsLayout ws_layout(int64_t r, int64_t c) {
     WsLayout L;
     L.ldc = lq_ceil_div(c, 4) * 4;
-    L.ldt = c > OB ? OB : lq_ceil_div(c, 8) * 8;
+    L.digits = c > OB && r * c >= DIGITS_MIN_WEIGHTS;
+    L.ldt = L.digits ? OB : lq_ceil_div(c, 8) * 8;
     size_t off = 0;
     L.wc = off; off += lq_align_up(static_cast<size_t>(r) * L.ldc * sizeof(float), 256);
     L.ut = off; off += lq_align_up(static_cast<size_t>(3) * c * L.ldt * sizeof(__nv_bfloat16), 256);
     L.es = off; off += lq_align_up(static_cast<size_t>(3) * r * OB * sizeof(__nv_bfloat16), 256);
     L.loss = off; off += lq_align_up(static_cast<size_t>(r) * sizeof(double), 256);
     L.ud = L.ed = L.cscale = L.rscale = off;
-    if (c > OB) {                          // the digits and scales of one outer block's errors and of the rows of U beside it
+    if (L.digits) {                        // the digits and scales of one outer block's errors and of the rows of U beside it
         L.ud = off; off += lq_align_up(static_cast<size_t>(FAR_SLICES) * c * OB, 256);
         L.ed = off; off += lq_align_up(static_cast<size_t>(FAR_SLICES) * r * OB, 256);
         L.cscale = off; off += lq_align_up(static_cast<size_t>(c + 256) * sizeof(float), 256);      // read up to the end of a tile
@@ -966,8 +971,8 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
         LQ_LAUNCH_CHECK();
     }
     if (c > B) {
-        dim3 g(static_cast<unsigned>(lq_ceil_div(c, 64)), static_cast<unsigned>(lq_ceil_div(L.ldt, 64)));      // the blocks on the diagonal
-        split_transpose_kernel<<<g, 256, 0, st>>>(U, ldu, c, UT, L.ldt);
+        dim3 g(static_cast<unsigned>(lq_ceil_div(c, 64)), static_cast<unsigned>(lq_ceil_div(L.ldt, 64)));
+        split_transpose_kernel<<<g, 256, 0, st>>>(U, ldu, c, UT, L.ldt, L.digits ? 1 : 0);
         LQ_LAUNCH_CHECK();
     }
     zero_doubles_kernel<<<static_cast<unsigned>(lq_ceil_div(r, 256)), 256, 0, st>>>(loss_rows, r);
@@ -1029,7 +1034,7 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
         if (near > 0) {
             lq_tc_gemm_args g = {};
             g.A_all = ES + (i0 - o0); g.a_rows = 3 * r; g.lda = OB;
-            g.B_all = UT + (i0 + B) * L.ldt + (i0 - o0); g.b_rows = 3 * c - (i0 + B); g.ldb = L.ldt;
+            g.B_all = UT + (i0 + B) * L.ldt + (i0 - (L.digits ? o0 : 0)); g.b_rows = 3 * c - (i0 + B); g.ldb = L.ldt;
             g.D = Wc + (i0 + B); g.ldd = L.ldc;
             g.M = r; g.N = near; g.K = B;
             g.n_pass = 6;
@@ -1039,7 +1044,20 @@ int quantize_impl(lq_handle* h, void* stream, const lq_config* cfg, const void* 
             if (rc) return rc;
         }
         if (i0 + B >= ob_end && ob_end < c) {
-            rc = affine ? far_update<4>(h, st, L, wsp, U, ldu, r, c, o0) : far_update<3>(h, st, L, wsp, U, ldu, r, c, o0);
+            if (L.digits) {
+                rc = affine ? far_update<4>(h, st, L, wsp, U, ldu, r, c, o0) : far_update<3>(h, st, L, wsp, U, ldu, r, c, o0);
+            } else {
+                lq_tc_gemm_args g = {};
+                g.A_all = ES; g.a_rows = 3 * r; g.lda = OB;
+                g.B_all = UT + ob_end * L.ldt + o0; g.b_rows = 3 * c - ob_end; g.ldb = L.ldt;
+                g.D = Wc + ob_end; g.ldd = L.ldc;
+                g.M = r; g.N = c - ob_end; g.K = ob_end - o0;
+                g.n_pass = 6;
+                for (int i = 0; i < 6; ++i) { g.a_row_off[i] = ao[i]; g.b_row_off[i] = bo[i]; }
+                g.alpha = -1.0f; g.accumulate = 1; g.upper_only = 0;
+                g.seg_iters = 12;          // partial sums leave the tensor core's truncating accumulator every 12 k-steps
+                rc = lq_tc_gemm(h, st, g);
+            }
             if (rc) return rc;
         }
     }

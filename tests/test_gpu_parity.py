@@ -541,6 +541,40 @@ def test_stage4_tall_layers_row_for_row(lq, h, c, bits, group, copies):
     np.testing.assert_allclose(out[1][2], out[0][2], rtol=1e-6)          # per block a row's fp32 sum of squares in another order
 
 
+@pytest.mark.parametrize("c,bits,group,r", [(2180, 3, 0, 11600), (2180, 4, 20, 11600), (3076, 2, 0, 8300)])
+def test_stage4_digit_products_against_the_oracle(lq, h, c, bits, group, r):
+    """Layers of 24 M weights and more take the errors beyond an outer block as products of 8-bit digits: copies of 50 rows
+    against the oracle's loop (ragged last tiles and blocks, both slice counts, both forms of the column loop); every copy of
+    a row gets the same codes, and a row with a NaN or an infinity keeps them to itself."""
+    n0 = 50
+    L = synth.make_layer("c3", n0, c, 2 * c, seed=c + bits)
+    W = f64(L.W)
+    U, dinv, _, _ = O.prepare_hinv(O.hessian(f64(L.X)), 0.01)
+    U32 = torch.from_numpy(U).float()
+    k = r // n0
+    if group:
+        So, Zo = O.fit_grid_affine(W, dinv, bits, 4.0, group, 20, 4)
+        S32, Z32 = torch.from_numpy(So).float(), torch.from_numpy(Zo).int()
+        kw, pts = dict(scale=f64(S32), zero=f64(Z32), group=group), aff_points(f64(S32), f64(Z32), 1 << bits, group, c)
+        gkw = dict(scale=S32.repeat(k, 1), zero=Z32.repeat(k, 1))
+        cfg = lq.Config.make(grid="affine", bits=bits, group=group, T=20, t=4)
+    else:
+        G32 = torch.from_numpy(O.fit_grid_nonuniform(W, dinv, bits, 4.0, 20)).float()
+        kw, pts = dict(grid=f64(G32)), nu_points(G32)
+        gkw = dict(grid=G32.repeat(k, 1))
+        cfg = lq.Config.make(grid="nonuniform", bits=bits)
+    codes_o, _, loss_o, Wpre = O.quantize_layer(W, f64(U32), bits=bits, block=128, return_pre=True, **kw)
+    Wk = L.W.repeat(k, 1)
+    codes, _, loss = run_stage4(lq, h, Wk, U32, cfg, **gkw)
+    codes = codes.reshape(k, n0, c)
+    assert (codes == codes[:1]).all()
+    codes_agree(codes[0], codes_o, Wpre, pts)
+    assert abs(loss / k / loss_o - 1) <= LOSS_TOL
+    Wk[0, 5], Wk[n0, 1500] = float("nan"), float("inf")
+    again, _, _ = run_stage4(lq, h, Wk, U32, cfg, **gkw)
+    assert (again.reshape(k, n0, c)[2:] == codes[:1]).all() and (again[1:n0] == codes[0, 1:]).all()
+
+
 @pytest.mark.parametrize("grid_type", ["nonuniform", "affine"])
 def test_stage4_many_rows_odd_count(lq, h, grid_type):
     """From 24 rows per SM on a warp of the in-block kernel carries two rows: an odd row count (the last warp has one
